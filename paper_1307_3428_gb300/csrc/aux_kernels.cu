@@ -9,6 +9,15 @@ namespace cme {
 
 namespace {
 
+// A complex factor of modulus <= 1 times 2^62 as balanced limbs (cme_fixed.cuh).
+__device__ int4 factor_limbs(double re, double im)
+{
+    const long long C = __double2ll_rn(re * 4611686018427387904.0);
+    const long long S = __double2ll_rn(im * 4611686018427387904.0);
+    return make_int4((int)((unsigned)(C >> 32) + ((unsigned)C >> 31)), (int)C,
+                     (int)((unsigned)(S >> 32) + ((unsigned)S >> 31)), (int)S);
+}
+
 __global__ void twiddle_kernel(int N, int prec, void* out)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -16,9 +25,9 @@ __global__ void twiddle_kernel(int N, int prec, void* out)
         return;
     double s, c;
     sincospi(2.0 * (double)k / (double)N, &s, &c);   // exp(2 pi i k/N) in FP64
-    if (prec == PREC_FP64)
-        reinterpret_cast<double2*>(out)[k] = make_double2(c, s);
-    else
+    if (prec == PREC_FP64) {
+        reinterpret_cast<int4*>(out)[k] = factor_limbs(c, s);
+    } else
         reinterpret_cast<float2*>(out)[k] = make_float2((float)c, (float)s);
 }
 
@@ -58,7 +67,10 @@ __global__ void prop_kernel(PropArgs a)
     const double2 e1 = cexpm1(Lr * hh, Li * hh);
     const double2 e2 = cexpm1(Lr * a.h, Li * a.h);
     put<V>(a.E, m, make_double2(e1.x + 1.0, e1.y));
-    put<V>(a.e1, m, e1);
+    if (a.e1)
+        put<V>(a.e1, m, e1);
+    if (a.Ef)
+        reinterpret_cast<int4*>(a.Ef)[m] = factor_limbs(e1.x + 1.0, e1.y);
     put<V>(a.e2, m, e2);
     // Strang pump increment over h/2 on the pumped mode (transform position 0):
     //   c = (exp(L_0 h/2) - 1) / L_0 * pump   (h/2 * pump when L_0 = 0)

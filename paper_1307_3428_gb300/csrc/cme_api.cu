@@ -188,7 +188,7 @@ struct cme_batch_s {
     std::vector<void*> allocs;
     cme_free_fn free_fn = nullptr;
     void* free_ctx = nullptr;
-    void *hi = nullptr, *lo = nullptr, *E = nullptr, *e1 = nullptr, *e2 = nullptr,
+    void *hi = nullptr, *lo = nullptr, *E = nullptr, *e1 = nullptr, *e2 = nullptr, *Ef = nullptr,
          *diag = nullptr;
     double *kappa = nullptr, *omega = nullptr, *sigma_d = nullptr, *g0_d = nullptr;
     double2 *pump_d = nullptr, *cpump_d = nullptr, *cpump2_d = nullptr, *stage = nullptr;
@@ -697,6 +697,8 @@ int cme_batch_create(const cme_instance* v, int count, const cme_options* opt, v
     b->E = A(T * b->elem);
     b->e1 = A(T * b->elem);
     b->e2 = A(T * b->elem);
+    if (b->prec == PREC_FP64 && b->method == METHOD_RK4IP)
+        b->Ef = A(T * 16);
     b->diag = A(T * b->elem);
     b->kappa = (double*)A(T * 8);
     b->omega = (double*)A(T * 8);
@@ -922,6 +924,7 @@ StepArgs group_args(cme_batch b, const LaunchGroup& g)
     a.E = b->E;
     a.e1 = b->e1;
     a.e2 = b->e2;
+    a.Ef = b->Ef;
     a.tw = b->tw[g.logN];
     a.pump = b->pump_d + g.first;
     a.cpump = b->cpump_d + g.first;
@@ -1207,6 +1210,7 @@ int ensure_propagators(cme_batch b, double h)
     p.prec = b->prec;
     p.E = b->E;
     p.e1 = b->e1;
+    p.Ef = b->Ef;
     p.e2 = b->e2;
     p.cpump = b->cpump_d;
     p.cpump2 = b->cpump2_d;

@@ -76,6 +76,18 @@ CME_DEV void store(void* p, long long i, cx<T> a)
     v.y = a.im;
     reinterpret_cast<typename v2<T>::type*>(p)[i] = v;
 }
+// A value that waits in global memory (this thread's own slot) and is read back by the same
+// thread; volatile, so that it does not stay in registers instead.
+CME_DEV void park_store(cx<double>* p, cx<double> v)
+{
+    asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.re), "d"(v.im) : "memory");
+}
+CME_DEV cx<double> park_load(const cx<double>* p)
+{
+    cx<double> v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "l"(p) : "memory");
+    return v;
+}
 
 // ----------------------------------------------------------------------------------------
 // Transform plan: N = 2^LOGN, R values per thread, NS passes, last radix 2^LOG_LAST.

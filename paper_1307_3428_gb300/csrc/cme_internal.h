@@ -21,6 +21,7 @@ struct StepArgs {
     const void* E;          // exp(L h/2) per mode                (RK4IP)
     const void* e1;         // expm1(L h/2) per mode              (RK4IP and Strang)
     const void* e2;         // expm1(L h) per mode                (RK4IP)
+    const void* Ef;         // FP64 RK4IP: limbs of E per mode (cme_fixed.cuh), else null
     const void* tw;         // twiddle table exp(2 pi i k / N), k < N
     const double2* pump;    // per-instance pump sqrt(kappa_ext) A_in (group-relative)
     const double2* cpump;   // per-instance Strang pump increment over h/2
@@ -73,9 +74,16 @@ __host__ __device__ constexpr size_t tw_bytes(int tbytes, int logN, int R)
                      ((1 << logN) / R) * 8
                : 0;
 }
+// FP64 groups wider than a warp: one (key, count) pair per warp for the scale of the fixed-point
+// transforms
+__host__ __device__ constexpr size_t red_bytes(int tbytes, int P)
+{
+    return tbytes == 8 && P > 32 ? (size_t)(P / 32) * 8 : 0;
+}
 __host__ __device__ constexpr size_t group_smem_bytes(int tbytes, int logN, int R)
 {
-    return xbuf_bytes(tbytes, logN) + acc_bytes(tbytes, logN, R) + tw_bytes(tbytes, logN, R);
+    return xbuf_bytes(tbytes, logN) + acc_bytes(tbytes, logN, R) + tw_bytes(tbytes, logN, R) +
+           red_bytes(tbytes, (1 << logN) / R);
 }
 
 // Cluster launches: one instance spread over the C blocks of a thread-block cluster.  Compiled
@@ -126,8 +134,9 @@ struct PropArgs {
     double h;
     int prec;
     void* E;
-    void* e1;
+    void* e1;                 // null: skipped
     void* e2;
+    void* Ef;                 // FP64 RK4IP: limbs of E (int4 per mode), null: skipped
     void* e1h;                // Strang: expm1(L h/2)
     double2* cpump;           // Strang pump increment per instance
     double2* cpump2;          // the same over h (null: not computed)

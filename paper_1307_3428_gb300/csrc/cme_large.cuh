@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(max_threads<LOGN2, R>()) large_row_kernel(cons
     cx<T> w[R];
 #pragma unroll
     for (int j = 0; j < R; ++j)
-        w[j] = gload<T>(A.twN, ((long long)j1 * (t + j * P)) & (N - 1));
+        w[j] = twload<T>(A.twN, ((long long)j1 * (t + j * P)) & (N - 1));
     pdl_wait();
     pdl_trigger();
     const cx<T>* yrow = reinterpret_cast<const cx<T>*>(A.Y) + ibase + (long long)t * N1 + j1;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(max_threads<LOGN1, R>()) large_col_kernel(cons
             else if (st == 2 || st == 3)
                 ev[j] = gload<T>(e2p, o);
             if (st != LARGE_FINAL)
-                w[j] = gload<T>(A.twN, ((long long)(t + j * P) * m2) & (N - 1));
+                w[j] = twload<T>(A.twN, ((long long)(t + j * P) * m2) & (N - 1));
         }
     }
     pdl_wait();
@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(Plan<LOGN1, R>::P) large_grid_kernel(const Lar
         Dh[j] = hi[j * PC];
         Dl[j] = COMP ? lo[j * PC] : cx<T>{T(0), T(0)};
         Sv[j] = cx<T>{T(0), T(0)};
-        wc[j] = gload<T>(A.twN, ((long long)(t + j * PC) * m2) & (N - 1));
-        wr[j] = gload<T>(A.twN, ((long long)j1 * (tr + j * PR)) & (N - 1));
+        wc[j] = twload<T>(A.twN, ((long long)(t + j * PC) * m2) & (N - 1));
+        wr[j] = twload<T>(A.twN, ((long long)j1 * (tr + j * PR)) & (N - 1));
     }
     const T gNr = (T)A.g0[ri] * ((T)1 / (T)N);
     T h, hh, h6;

@@ -129,7 +129,7 @@ extern "C" int cme_rk4ip_noalloc(int N, int count, double h, long nsteps, const 
     Carver cv{(unsigned char*)base};
     double2* hi = (double2*)cv.take(total * 16);
     void* E = cv.take(total * 16);
-    void* e1 = cv.take(total * 16);
+    void* Ef = cv.take(total * 16);
     void* e2 = cv.take(total * 16);
     double* kappa_t = (double*)cv.take(total * 8);
     double* omega_t = (double*)cv.take(total * 8);
@@ -165,7 +165,7 @@ extern "C" int cme_rk4ip_noalloc(int N, int count, double h, long nsteps, const 
         p.h = h;
         p.prec = PREC_FP64;
         p.E = E;
-        p.e1 = e1;
+        p.Ef = Ef;
         p.e2 = e2;
         p.cpump = cpump;
         p.ninst = count;
@@ -193,7 +193,7 @@ extern "C" int cme_rk4ip_noalloc(int N, int count, double h, long nsteps, const 
         a.hi = hi;
         a.lo = nullptr;
         a.E = E;
-        a.e1 = e1;
+        a.Ef = Ef;
         a.e2 = e2;
         a.tw = tw;
         a.pump = pump;

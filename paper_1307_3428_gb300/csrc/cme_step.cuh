@@ -5,6 +5,7 @@
 #include <type_traits>
 
 #include "cme_core.cuh"
+#include "cme_fixed.cuh"
 
 namespace cme {
 
@@ -27,6 +28,7 @@ struct Props {
     const cx<T>* pE;   // pointers pre-offset to (instance offset + t)
     const cx<T>* pe1;
     const cx<T>* pe2;
+    const int4* pF;    // FP64: limbs of E (StepArgs::Ef)
 
     CME_DEV void init(const StepArgs& a, long long off, int t)
     {
@@ -34,6 +36,7 @@ struct Props {
         pE = reinterpret_cast<const cx<T>*>(a.E) + off + t;
         pe1 = reinterpret_cast<const cx<T>*>(a.e1) + off + t;
         pe2 = reinterpret_cast<const cx<T>*>(a.e2) + off + t;
+        pF = reinterpret_cast<const int4*>(a.Ef) + off + t;
         if constexpr (IN_REGS) {
 #pragma unroll
             for (int j = 0; j < R; ++j) {
@@ -43,6 +46,7 @@ struct Props {
             }
         }
     }
+    CME_DEV fl2 getF(int j) const { return fx_twiddle(pF, j * Plan<LOGN, R>::P); }
     CME_DEV cx<T> getE(int j) const
     {
         if constexpr (IN_REGS)
@@ -83,6 +87,9 @@ struct GroupFFT<T, LOGN, R, 1> {
     using TF = Transform<T, LOGN, R, (Plan<LOGN, R>::P <= 32)>;
 };
 
+template <typename T, int LOGN, int R, int C>
+CME_HD constexpr size_t cluster_smem_bytes();
+
 // Per-thread view of one instance: the transform machinery plus the instance constants.
 // C > 1: the instance is spread over the C blocks of a thread-block cluster.
 template <typename T, int LOGN, int R, int C = 1>
@@ -100,8 +107,14 @@ struct Group {
     static constexpr bool TW_REGS =
         twiddles_in_regs<T, LOGN - LC>() && (C == 1 || sizeof(T) == 4);
     static constexpr bool TW_SMEM = !TW_REGS && twiddles_in_smem(sizeof(T), LOGN - LC);
-    using TW = std::conditional_t<TW_SMEM, TwiddlesSmem<T, LOGN - LC, R, C>,
-                                  Twiddles<T, LOGN - LC, R, TW_REGS, C>>;
+    // FP64 transforms run in fixed point (cme_fixed.cuh)
+    static constexpr bool FIX = sizeof(T) == 8;
+    using FT = FixTransform<LOGN - LC, R, (Plan<LOGN - LC, R>::P <= 32)>;
+    using TW = std::conditional_t<
+        FIX, FixTwiddles<LOGN - LC, R, TW_REGS, C>,
+        std::conditional_t<TW_SMEM, TwiddlesSmem<T, LOGN - LC, R, C>,
+                           Twiddles<T, LOGN - LC, R, TW_REGS, C>>>;
+    int2* red;     // FP64: reduction pairs of this group's warps (shared memory)
 
     int t;         // the thread holds modes t + jP
     int ts;        // this thread's slots ts + jP of per-thread scratch vectors (coalesced)
@@ -194,19 +207,34 @@ struct Group {
     CME_DEV void inverse(cx<T> (&x)[R], int d)
     {
         if constexpr (C == 1) {
-            TF::template run<+1>(x, tw, buf, par, ad);
+            block_inverse(x);
         } else {
             if (d == 1) {
                 CF::radix_c(x);
                 twiddle(x, twt);
                 all_to_all<true>(x);
             }
-            TF::template run<+1>(x, tw, buf, par, ad);
+            block_inverse(x);
             if (d == 0) {
                 twiddle(x, twm);
                 all_to_all<false>(x);
                 CF::radix_c(x);
             }
+        }
+    }
+    // this thread's index among those that share a transform's block
+    CME_DEV int tl() const { return C == 1 ? t : (int)threadIdx.x; }
+    // the inverse transform inside one block
+    CME_DEV void block_inverse(cx<T> (&x)[R])
+    {
+        if constexpr (FIX) {
+            fx X[R];
+            const typename FT::Scale sc = FT::load(x, X, red, tl());
+            const typename FT::Shifts h = FT::shifts(sc.b);
+            FT::run(X, tw, buf, par, ad, h);
+            FT::store(X, h.cur - sc.q, x);
+        } else {
+            TF::template run<+1>(x, tw, buf, par, ad);
         }
     }
     CME_DEV static void twiddle(cx<T> (&x)[R], const cx<T>* w)
@@ -259,6 +287,44 @@ struct Group {
     // The same, also storing the time-domain field a at aout[j P] unless aout is null.
     CME_DEV void rhs_store_a(cx<T> (&x)[R], T gN, cx<T> pump, cx<T>* aout)
     {
+        if constexpr (FIX && C == 1)
+            fix_rhs(x, gN, aout);
+        else
+            float_rhs(x, gN, aout);
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            x[j].im = -x[j].im;
+        out_modes(x);
+        if (t == 0)
+            x[0] = cadd(x[0], pump);
+    }
+    // x becomes conj(i gN DFT(|a|^2 a)): both transforms and the Kerr term in fixed point
+    CME_DEV void fix_rhs(cx<T> (&x)[R], T gN, cx<T>* aout)
+    {
+        fx X[R];
+        const typename FT::Scale sc = FT::load(x, X, red, tl());
+        typename FT::Shifts h = FT::shifts(sc.b);
+        int q = sc.q;
+#pragma unroll 1
+        for (int d = 0; d < 2; ++d) {
+            FT::run(X, tw, buf, par, ad, h);
+            q -= h.cur;
+            if (d == 0) {
+                if (aout) {
+                    FT::store(X, -q, x);
+#pragma unroll
+                    for (int j = 0; j < R; ++j)
+                        sstore(aout + j * P, x[j]);
+                }
+                const typename FT::Kerr k = FT::kerr(X, q, gN, red, tl());
+                q = k.q;
+                h = FT::shifts(k.b);
+            }
+        }
+        FT::store(X, -q, x);
+    }
+    CME_DEV void float_rhs(cx<T> (&x)[R], T gN, cx<T>* aout)
+    {
 #pragma unroll 1
         for (int d = 0; d < 2; ++d) {
             inverse(x, d);
@@ -276,12 +342,6 @@ struct Group {
                 }
             }
         }
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-            x[j].im = -x[j].im;
-        out_modes(x);
-        if (t == 0)
-            x[0] = cadd(x[0], pump);
     }
 
     static constexpr bool ACC_SMEM = C == 1 && acc_in_smem(sizeof(T), LOGN, R);
@@ -298,6 +358,8 @@ struct Group {
         static_assert(xbuf_bytes(sizeof(T), LOGN) == (size_t)2 * W * PL::BUF * 8, "layout");
         accS = acc + t_;
         accL = acc + N + t_;
+        red = reinterpret_cast<int2*>(gbase + xbuf_bytes(sizeof(T), LOGN) +
+                                      acc_bytes(sizeof(T), LOGN, R) + tw_bytes(sizeof(T), LOGN, R));
         if constexpr (sizeof(T) == 4) {
             buf.p = reinterpret_cast<float2*>(base);
         } else {
@@ -321,8 +383,8 @@ struct Group {
     // Cluster set-up (C > 1): block `rank` of the cluster, thread l of the block.  The block's
     // dynamic shared memory holds the two exchange buffers of its N2-point transform, the two
     // all-to-all receive buffers, the two twiddle arrays of the four-step transform, (FP32,
-    // N2 >= 2048) the pass twiddles of the N2-point transform, and the receive buffers' two
-    // mbarriers (its last 16 bytes).
+    // N2 >= 2048) the pass twiddles of the N2-point transform, the receive buffers' two
+    // mbarriers and (FP64) the reduction pairs.
     CME_DEV void setup_cluster(unsigned char* smem, int rank, int l, const void* tw_table,
                                int a2a_fault)
     {
@@ -358,6 +420,8 @@ struct Group {
             rb[c] = dsmem_map(a0, c);
             rmb[c] = dsmem_map(mb, c);
         }
+        red = reinterpret_cast<int2*>(smem + cluster_smem_bytes<T, LOGN, R, C>() -
+                                      red_bytes(sizeof(T), PC));
         // the kernel's cluster barrier before the first all-to-all publishes the initialisation
         if (l == 0) {
             mbar_init(mb, 1);
@@ -376,8 +440,8 @@ struct Group {
         cx<T>* wt = tws + N2 + l;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            wm[j * PC] = gload<T>(tw_table, ((l + PC * j) * rank) & (N - 1));
-            wt[j * PC] = gload<T>(tw_table, ((tp + P * (j % G)) * (j / G)) & (N - 1));
+            wm[j * PC] = twload<T>(tw_table, ((l + PC * j) * rank) & (N - 1));
+            wt[j * PC] = twload<T>(tw_table, ((tp + P * (j % G)) * (j / G)) & (N - 1));
         }
         twm = wm;
         twt = wt;
@@ -386,7 +450,7 @@ struct Group {
     }
 };
 
-// Dynamic shared memory of one block of a cluster group: two exchange buffers.
+// Dynamic shared memory of one block of a cluster group (Group::setup_cluster).
 template <typename T, int LOGN, int R, int C>
 CME_HD constexpr size_t cluster_smem_bytes()
 {
@@ -394,7 +458,8 @@ CME_HD constexpr size_t cluster_smem_bytes()
     constexpr size_t W = Xbuf<T>::words_per_elem;
     return (size_t)2 * CF::TL::BUF * 8 * W + (size_t)2 * CF::N2 * 8 * W +
            (size_t)2 * CF::N2 * sizeof(cx<T>) +
-           (Group<T, LOGN, R, C>::TW_SMEM ? tw_bytes(sizeof(T), LOGN - CF::LC, R) : 0) + 16;
+           (Group<T, LOGN, R, C>::TW_SMEM ? tw_bytes(sizeof(T), LOGN - CF::LC, R) : 0) + 16 +
+           red_bytes(sizeof(T), CF::PC);
 }
 
 template <typename T>
@@ -602,6 +667,175 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
     }
 }
 
+// One RK4IP step of an FP64 one-block group with the stages in fixed point (cme_fixed.cuh).  The
+// state D, its propagation and the step's increment are FP64; what only enters a right-hand side
+// (the stage inputs) or the increment (the right-hand sides and their sum) stays in fixed
+// point, each on its own block scale, as in
+//     Y1 = h/2 F(D),    U = E D,  A = E Y1,   x2 = U + A,
+//     Y2 = h/2 F(x2),   A += 2 Y2,            x3 = U + Y2,
+//     Y3 = h F(x3),     A += Y3,              x4 = E (U + Y3),
+//     Y4 = h/2 F(x4),   D' = D + [expm1(L h) D + (E A + Y4) / 3],
+// the same step as rk4ip_step_impl.  Per mode and step that leaves 8 FP64 instructions of the 74
+// outside the transforms, and one conversion from and one to FP64 instead of four each.
+// N = 512 x 256: 88.5 us per step with FP64 instructions throughout (bound by their pipe), 36.8
+// with only the transforms and the Kerr term in fixed point, 23.0 with the stages.  One N = 64
+// instance: 19.5, 11.7 and 7.7 us.  What bounds it now is one warp per scheduler issuing dependent
+// integer instructions (fixed-latency waits, 1.4 per issue).
+// The error of a step against extended precision on the small modes of a comb (1e-6 beside a
+// pumped mode of 1.3, h = 2e-4): 1.3e-21 at N = 512 and 1.4e-21 at 4096, from 4.9e-21 and 1.6e-21
+// in FP64 instructions.  It is set by the units of the stage inputs and of the increment, so both
+// keep every bit the bounds leave (fcmul1, not fcmul4, there).
+// park: where the state waits in global memory during the step (groups whose registers and shared
+// memory are full: ACC_SMEM), else unused.  STAGES: as in rk4ip_step_impl.
+template <bool STAGES, int LOGN, int R>
+CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, LOGN, R, 1>& fs,
+                            const Props<double, LOGN, R, 1>& pr, const StepConsts<double>& c,
+                            cx<double>* park, cx<double>* so, long long sstride)
+{
+    using GR = Group<double, LOGN, R, 1>;
+    using FT = typename GR::FT;
+    constexpr int P = GR::P;
+    constexpr bool AS = GR::ACC_SMEM;
+    fx X[R], U[R], Ar[AS ? 1 : R];
+    auto getA = [&](int j) -> fx {
+        if constexpr (AS) {
+            const cx<double> v = grp.accS[j * P];
+            return {__double_as_longlong(v.re), __double_as_longlong(v.im)};
+        } else {
+            return Ar[j];
+        }
+    };
+    auto setA = [&](int j, fx v) {
+        if constexpr (AS)
+            grp.accS[j * P] = {__longlong_as_double(v.re), __longlong_as_double(v.im)};
+        else
+            Ar[j] = v;
+    };
+    const typename FT::Scale sc = FT::load(fs.Dh, X, grp.red, grp.tl());
+    if constexpr (AS) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            park_store(park + j * P, fs.Dh[j]);
+    }
+    const bool bad = sc.q == FT::POISON;
+    FixBound b = sc.b;
+    int q = bad ? 0 : sc.q, bY = 0, qU = q, bU = min(b.bm, b.bl), qA = 0, bA = 0;
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        U[j] = X[j];
+    const double gh = c.gN * c.hh;
+    const cx<double> pump = cscale(c.pump, c.hh);
+    // |pump| < 2^eP
+    const int eP = (int)(max(FT::habs(pump.re), FT::habs(pump.im)) >> 20) - 1022 + 1;
+#pragma unroll 1
+    for (int st = 0; st < 4; ++st) {
+        typename FT::Shifts h = FT::shifts(b);
+        // X becomes Y of this stage, scale q, modulus below 2^bY
+#pragma unroll 1
+        for (int d = 0; d < 2; ++d) {
+            FT::run(X, grp.tw, grp.buf, grp.par, grp.ad, h);
+            q -= h.cur;
+            if (d == 0) {
+                if constexpr (STAGES) {
+                    if (so) {
+                        cx<double> a[R];
+                        FT::store(X, bad ? -FT::POISON : -q, a);
+#pragma unroll
+                        for (int j = 0; j < R; ++j)
+                            sstore(so + (3 + st) * sstride + j * P, a[j]);
+                    }
+                }
+                const typename FT::Kerr k = FT::kerr(X, q, gh, grp.red, grp.tl());
+                q = k.q - (st == 2);
+                b = k.b;
+                h = FT::shifts(b);
+            } else {
+                bY = min(b.bl, b.bm + LOGN) - h.cur;
+            }
+        }
+        // the sum with the pump stays below 2^62
+        const int s = max(eP + (st == 2) + q, bY) - 61;
+        if (s > 0) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                X[j] = {frsh(X[j].re, min(s, 63)), frsh(X[j].im, min(s, 63))};
+            q -= s;
+            bY -= s;
+        }
+        bY = max(bY, eP + (st == 2) + q) + 1;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            X[j].im = -X[j].im;
+            if (!grp.physical(j))
+                X[j] = {0, 0};
+        }
+        if (grp.t == 0) {
+            const int c0 = 1085 - q - (st == 2);
+            X[0] = fadd(X[0], {FT::fix(pump.re, c0), FT::fix(pump.im, c0)});
+        }
+        if constexpr (STAGES) {
+            if (so && st < 3) {
+                cx<double> y[R];
+                FT::store(X, bad ? -FT::POISON : -q, y);
+                const double ih = 1.0 / (st == 2 ? c.h : c.hh);
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    sstore(so + st * sstride + j * P, cscale(y[j], ih));
+            }
+        }
+        if (st == 3)
+            break;
+        if (st == 0) {
+            qA = q - 2;
+            bA = bY - 2;
+            const typename FT::Align al = FT::align(qU, bU, qA, bA);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const fl2 E = pr.getF(j);
+                const fx a = fcmul4(X[j], E, 0);
+                U[j] = fcmul1(U[j], E);
+                setA(j, a);
+                X[j] = FT::asum(U[j], a, al);
+            }
+            q = al.q;
+        } else {
+            // A += (2 or 1) Y
+            const typename FT::Align aa = FT::align(qA, bA, q - (st == 1), bY);
+            bA = max(bA - (qA - aa.q), bY - (q - (st == 1) - aa.q)) + 1;
+            qA = aa.q;
+            const typename FT::Align al = FT::align(qU, bU, q, bY);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                setA(j, FT::asum(getA(j), X[j], aa));
+                X[j] = FT::asum(U[j], X[j], al);
+            }
+            q = al.q;
+            if (st == 2)
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    X[j] = fcmul1(X[j], pr.getF(j));
+        }
+        b = FT::bounds(X, grp.red, grp.tl());
+        q += FT::rescale(X, b);
+    }
+    // the increment (E A + Y4) / 3
+    // (unscaled product: the increment's unit, relative to its largest mode, is what limits the
+    // accuracy of the small ones)
+    const typename FT::Align al = FT::align(qA, bA, q, bY);
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        X[j] = FT::asum(fcmul1(getA(j), pr.getF(j)), X[j], al);
+    cx<double> w[R];
+    FT::store(X, bad ? -FT::POISON : -al.q, w);
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        if constexpr (AS)
+            fs.Dh[j] = park_load(park + j * P);
+        const cx<double> d = cmul(pr.get2(j), fs.Dh[j]);
+        fs.Dh[j] = cadd(fs.Dh[j], caxpy(d, 1.0 / 3.0, w[j]));
+    }
+}
+
 // Whether a step kernel has the registers to keep e1 D / e2 D across a stage (FP32 at 8 values
 // per thread, at most 256 threads per block: N = 512, 64 threads, 168 -> 192 registers), not
 // in the work-list kernel, whose tiles share one register budget.
@@ -616,6 +850,22 @@ CME_DEV void rk4ip_step(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C>& fs
                         const Props<T, LOGN, R, C>& pr, const StepConsts<T>& c)
 {
     rk4ip_step_impl<false, CACHE>(grp, fs, pr, c, static_cast<cx<T>*>(nullptr), 0);
+}
+
+// The RK4IP step of a one-block group: FP64 in fixed point, except with per-mode Kerr factors (of
+// any size, so without a common scale).
+template <bool STAGES, bool CACHE, typename T, int LOGN, int R>
+CME_DEV void block_rk4ip_step(Group<T, LOGN, R, 1>& grp, FieldState<T, LOGN, R, 1>& fs,
+                              const Props<T, LOGN, R, 1>& pr, const StepConsts<T>& c, cx<T>* park,
+                              cx<T>* so, long long sstride)
+{
+    if constexpr (sizeof(T) == 8) {
+        if (!grp.km) {
+            fix_rk4ip_step<STAGES>(grp, fs, pr, c, park, so, sstride);
+            return;
+        }
+    }
+    rk4ip_step_impl<STAGES, CACHE>(grp, fs, pr, c, so, sstride);
 }
 
 // sin y and cos y in FP32 for the Strang Kerr phase y = g0 |a|^2 h / 2, which is small in any
@@ -804,7 +1054,8 @@ CME_DEV void step_body(const StepArgs& a, int first, unsigned char* smem)
 
     if constexpr (METHOD == METHOD_RK4IP) {
         for (long long n = 0; n < a.nsteps; ++n)
-            rk4ip_step<!FUSED && rk_cache_ed<T, LOGN, R, 1>()>(grp, fs, pr, c);
+            block_rk4ip_step<false, !FUSED && rk_cache_ed<T, LOGN, R, 1>()>(
+                grp, fs, pr, c, hi, static_cast<cx<T>*>(nullptr), 0);
     } else {
         const long long m = a.single_steps ? 1 : a.nsteps;
         for (long long n = 0; n < a.nsteps; n += m)
@@ -905,9 +1156,19 @@ __global__ void __launch_bounds__(max_threads<LOGN, R>()) diag_kernel(const Step
     for (int j = 0; j < R; ++j)
         x[j] = src[j * P];
     if (a.diag_mode == DIAG_IDFT) {
-        GR::TF::template run<+1>(x, grp.tw, grp.buf, grp.par, grp.ad);
+        grp.inverse(x, 0);
     } else if (a.diag_mode == DIAG_DFT) {
-        GR::TF::template run<-1>(x, grp.tw, grp.buf, grp.par, grp.ad);
+        if constexpr (GR::FIX) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                x[j].im = -x[j].im;
+            grp.inverse(x, 1);
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                x[j].im = -x[j].im;
+        } else {
+            GR::TF::template run<-1>(x, grp.tw, grp.buf, grp.par, grp.ad);
+        }
     } else {
         const double2 pd = a.pump[inst];
         grp.rhs(x, (T)(a.g0[inst] / (double)N), cx<T>{(T)pd.x, (T)pd.y});

@@ -248,6 +248,14 @@ struct FixTwiddles {
     }
 };
 
+// (-1)^n / (2n + 1)! and (-1)^n / (2n + 2)!, times 2^62: sin(x)/x and (1 - cos(x))/x^2 in x^2
+static __constant__ long long fx_sinc[10] = {
+    4611686018427387904, -768614336404564651, 38430716820228233, -915017067148291, 12708570377060,
+    -115532457973, 740592679, -3526632, 12966, -38};
+static __constant__ long long fx_cosc[10] = {
+    2305843009213693952, -192153584101141163, 6405119470038039, -114377133393536, 1270857037706,
+    -9627704831, 52899477, -220414, 720, -2};
+
 // Bounds of a group's values in bits: every value's modulus is below 2^bm, L1 below 2^bl.
 struct FixBound {
     int bm, bl;
@@ -490,15 +498,17 @@ struct FixTransform {
         }
     }
 
-    // Kerr term of the time samples a = X 2^-q: X becomes conj(i g |a|^2 a) 2^-k', with the
-    // scale k' returned for the next transform.  The samples are first scaled by their own
-    // largest modulus (they lie up to sqrt(N) below the bound of the transform), and L1 of
-    // the product comes from the same reduction.
+    // Scales of the Kerr term of the time samples a = X 2^-q with the coefficient g.  The samples
+    // are first scaled by their own largest modulus (they lie up to sqrt(N) below the bound of
+    // the transform), and L1 of the product comes from the same reduction.
     struct Kerr {
-        int q;
+        int up, us;   // left shifts of the samples and of the products g |a|^2
+        fl G;         // limbs of -g 2^(62 - eg), |g| = m 2^eg with m in [1/2, 1)
+        int qc;       // -g |a|^2 is (|a|^2 G) 2^-qc before its shift
+        int q;        // scale and bounds of conj(i g |a|^2 a)
         FixBound b;
     };
-    CME_DEV static Kerr kerr(fx (&X)[R], int q, double g, int2* red, int t)
+    CME_DEV static Kerr kerr_scale(const fx (&X)[R], int q, double g, int2* red, int t)
     {
         float mx = 0.f, f = 0.f;
 #pragma unroll
@@ -513,12 +523,12 @@ struct FixTransform {
         unsigned cnt = GRd::sum(
             (unsigned)(f * __int_as_float((127 + 12 - 3 * (key >> 1)) << 23)) + 1u);
         GRd::template combine<3, 1>(key, cnt, red, t);
-        const int up = max(61 - 40 - (key >> 1), 0);   // modulus below 2^61
+        Kerr k;
+        k.up = max(61 - 40 - (key >> 1), 0);   // modulus below 2^61
         // |a|^2 < 2^62, times |g| 2^(62 - eg) < 2^62 and a < 2^61: products below 2^57, and
         // below 2^KB with the product of |a|^2 and g shifted left by us; an even key leaves
         // |a|^2 one bit below its bound
-        const int us = KB - 57 + ((key & 1) ^ 1);
-        // |g| = m 2^eg, m in [1/2, 1): limbs of g 2^(62 - eg)
+        k.us = KB - 57 + ((key & 1) ^ 1);
         const int gh = __double2hiint(g);
         const int ge = (gh >> 20) & 0x7ff, eg = ge ? ge - 1022 : 0;
         const long long gm =
@@ -526,17 +536,87 @@ struct FixTransform {
                               (unsigned)__double2loint(g))
                              << 9)
                : 0;
-        const fl G = fsplit(gh < 0 ? gm : -gm);   // -g
+        k.G = fsplit(gh < 0 ? gm : -gm);
+        const int qa = q + k.up;
+        k.qc = 2 * qa - 62 - eg;
+        k.q = 3 * qa - 126 + k.us - eg;
+        k.b = {KB, KB + 32 - __clz((int)cnt) - 12};
+        return k;
+    }
+    // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc
+    CME_DEV static long long kerr_term(fx& X, const Kerr& k)
+    {
+        const fl r = fsplit(X.re << k.up), i = fsplit(X.im << k.up);
+        const long long m = fmad(i.h, i.l, fmad(r.h, r.l, 0x40000000LL));
+        const long long p2 = fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)) << 4;
+        const long long pg = fmulhi(fsplit(p2), k.G);
+        const fl c = fsplit(pg << k.us);
+        X = {fmulhi(c, i), fmulhi(c, r)};
+        return pg;
+    }
+    CME_DEV static Kerr kerr(fx (&X)[R], int q, double g, int2* red, int t)
+    {
+        const Kerr k = kerr_scale(X, q, g, red, t);
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const fl r = fsplit(X[j].re << up), i = fsplit(X[j].im << up);
-            const long long m = fmad(i.h, i.l, fmad(r.h, r.l, 0x40000000LL));
-            const long long p2 = fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)) << 4;
-            const fl c = fsplit(fmulhi(fsplit(p2), G) << us);
-            X[j] = {fmulhi(c, i), fmulhi(c, r)};
+        for (int j = 0; j < R; ++j)
+            kerr_term(X[j], k);
+        return k;
+    }
+    // The exact Kerr flow's increment: X becomes conj(a expm1(i phi)) / N, phi = gh |a|^2, for
+    // the next transform (scale k.q, bounds k.b).  For phi < 1 everywhere in the group
+    // expm1(i phi) = i phi F with the Taylor series F = sin(phi)/phi + i (1 - cos(phi))/phi in
+    // phi^2, cut where the group's largest phi leaves less than 2^-62 (5 terms at 0.06); larger
+    // phases take sincos in FP64 (no reduction in that branch: groups of a block may differ).
+    // 4 x N = 256 at 4 values per thread: 9.1 -> 5.0 us per split step, most of it the FP64
+    // instructions of sincos (about 3500 cycles per value, against about 350).
+    CME_DEV static Kerr kerr_flow(fx (&X)[R], int q, double gh, int2* red, int t)
+    {
+        constexpr double invN = 1.0 / N;
+        Kerr k = kerr_scale(X, q, gh * invN, red, t);
+        const int sh = k.qc - 62 - LOGN;   // |pg| < 2^60: phi 2^62 = |pg| 2^-sh < 2^(60 - sh)
+        if (sh >= -2) {
+            const int terms = sh < 0 ? (sh == -1 ? 8 : 10) : sh < 2 ? 7 : sh < 4 ? 5 : sh < 8 ? 4
+                              : sh < 15 ? 3 : 2;
+            const int rs = min(max(sh, 0), 63), ls = max(-sh, 0);
+            fx S[R];
+            long long ph[R];
+            fl z[R];
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                ph[j] = ((-kerr_term(X[j], k)) << ls) >> rs;
+                const fl p = fsplit(ph[j]);
+                z[j] = fsplit(fmulhi(p, p) << 2);
+                S[j] = {0, 0};
+            }
+#pragma unroll 1
+            for (int n = terms - 1; n >= 0; --n) {
+                const long long cs = fx_sinc[n], cc = fx_cosc[n];
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    S[j] = {cs + (fmulhi(fsplit(S[j].re), z[j]) << 2),
+                            cc + (fmulhi(fsplit(S[j].im), z[j]) << 2)};
+            }
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const long long im = fmulhi(fsplit(S[j].im), fsplit(ph[j])) << 2;
+                X[j] = fcmul1(X[j], {fsplit(S[j].re), fsplit(-im)});
+            }
+        } else {
+            cx<double> a[R];
+            store(X, -q, a);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                double sn, cs;
+                sincos(0.5 * gh * (a[j].re * a[j].re + a[j].im * a[j].im), &sn, &cs);
+                // conj(expm1(i phi)) / 4 as limbs; the product with a, 2^-5 of it
+                const fl2 w = {fsplit(fix(-sn * sn, 1085 - 61)), fsplit(fix(-sn * cs, 1085 - 61))};
+                const fx c = {X[j].re << k.up, -(X[j].im << k.up)};
+                X[j] = fcmul4(c, w, 1);
+            }
+            k.q = q + k.up - 5 + LOGN;
+            k.b = {61 - 4, 61 - 4 + LOGN};
         }
-        const int qa = q + up;
-        return {3 * qa - 126 + us - eg, {KB, KB + 32 - __clz((int)cnt) - 12}};
+        return k;
     }
     // Bounds of values that are below 2^62: the largest component and L1, from their high words.
     CME_DEV static FixBound bounds(const fx (&X)[R], int2* red, int t)

@@ -900,6 +900,51 @@ CME_DEV void strang_linear(const Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, 
     }
 }
 
+// The same in fixed point (FP64 one-block groups): both transforms, the phase and its exponential.
+template <bool STORE, int LOGN, int R>
+CME_DEV void fix_strang_kerr(Group<double, LOGN, R, 1>& grp, FieldState<double, LOGN, R, 1>& fs,
+                             const StepConsts<double>& c, cx<double>* so, long long sstride)
+{
+    using GR = Group<double, LOGN, R, 1>;
+    using FT = typename GR::FT;
+    constexpr int P = GR::P;
+    fx X[R];
+    cx<double> x[R];
+    const typename FT::Scale sc = FT::load(fs.Dh, X, grp.red, grp.tl());
+    typename FT::Shifts h = FT::shifts(sc.b);
+    int q = sc.q;
+#pragma unroll 1
+    for (int d = 0; d < 2; ++d) {
+        FT::run(X, grp.tw, grp.buf, grp.par, grp.ad, h);
+        q -= h.cur;
+        if (d == 0) {
+            if constexpr (STORE) {
+                if (so) {
+                    FT::store(X, -q, x);
+#pragma unroll
+                    for (int j = 0; j < R; ++j)
+                        sstore(so + j * P, x[j]);
+                }
+            }
+            const typename FT::Kerr k = FT::kerr_flow(X, q, 2.0 * c.g0h, grp.red, grp.tl());
+            q = k.q;
+            h = FT::shifts(k.b);
+        }
+    }
+    FT::store(X, -q, x);
+    grp.mask(x);   // no Kerr increment on padding modes
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        fs.add(j, cx<double>{x[j].re, -x[j].im});
+    if constexpr (STORE) {
+        if (so) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                sstore(so + sstride + j * P, fs.Dh[j]);
+        }
+    }
+}
+
 // Exact Kerr flow of the Strang step over h.  With a = inverse transform of D the flow is
 // a -> a exp(i g0 |a|^2 h); it is applied as the increment D += DFT(a expm1(i g0 |a|^2 h))/N.
 // STORE = true also stores, unless so is null (the adjoint's recomputation), the time-domain
@@ -908,6 +953,9 @@ template <bool STORE, typename T, int LOGN, int R, int C>
 CME_DEV void strang_kerr(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C>& fs,
                          const StepConsts<T>& c, cx<T>* so, long long sstride)
 {
+    if constexpr (sizeof(T) == 8 && C == 1) {
+        fix_strang_kerr<STORE>(grp, fs, c, so, sstride);
+    } else {
     constexpr int P = Group<T, LOGN, R, C>::P;
     constexpr T invN = (T)(1.0 / (1 << LOGN));
     cx<T> x[R];
@@ -967,6 +1015,7 @@ CME_DEV void strang_kerr(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C>& f
             for (int j = 0; j < R; ++j)
                 sstore(so + sstride + j * P, fs.Dh[j]);
         }
+    }
     }
 }
 

@@ -102,3 +102,48 @@ def test_non_finite_fields_are_reported(N, bad):
     b.set_state(D)
     b.step(1e-3, 3)
     assert b.status()[0] == 1
+
+
+def strang_extended(D, h, n, sigma=1.0, g0=1.3, pump=np.sqrt(L(0.5)) * L(0.7)):
+    """n Strang steps in extended precision (kappa = 1, omega = 0)."""
+    N = D.size
+    Lm = L(-0.5) - 1j * L(sigma)
+    half = np.exp(Lm * L(h) / 2)
+    x = np.fft.ifftshift(D.astype(L))
+    for _ in range(n):
+        x = half * x
+        x[0] += (half - 1) / Lm * pump
+        a = np.fft.ifft(x) * N
+        x = np.fft.fft(a * np.exp(1j * L(g0) * L(h) * (a.real ** 2 + a.imag ** 2))) / N
+        x = half * x
+        x[0] += (half - 1) / Lm * pump
+    return np.fft.fftshift(x)
+
+
+@pytest.mark.parametrize("N,R", [(4, 4), (16, 16), (64, 2), (64, 4), (256, 4), (512, 8), (4096, 8)])
+@pytest.mark.parametrize("phase", [1e-9, 1e-4, 0.03, 0.2, 0.45, 0.97, 1.1, 7.0])
+def test_split_step_phases(N, R, phase):
+    """Kerr phases from far below to above the Taylor series' range (1), on fields whose largest
+    sample has that phase.  Per step the linear flows round each mode three times and the Kerr
+    flow is one right-hand side."""
+    h = 1e-2
+    for name, D in fields(N).items():
+        a = np.fft.ifft(np.fft.ifftshift(D)) * N
+        D = D * np.sqrt(phase / (1.3 * h)) / np.abs(a).max()
+        b = batch(D, radix=R, integrator=cme.STRANG)
+        b.step(h, 2)
+        assert rel(b.get_state(), strang_extended(D, h, 2)) <= ULP * 8 * (np.log2(N) + 4), name
+        b.close()
+
+
+def test_split_step_phases_of_one_block_scale_apart():
+    D = [fields(64)["random"] * s for s in (1.0, 1e-3, 30.0, 1e-200, 0.0)]
+    insts = [cme.Instance(64, np.ones(64), np.zeros(64), 1.3, 0.5, 0.7, 1.0, d) for d in D]
+    kw = dict(radix=8, integrator=cme.STRANG)
+    b = cme.Batch(insts, **kw)
+    b.step(1e-2, 3)
+    together = b.get_state().reshape(len(D), 64)
+    for i, inst in enumerate(insts):
+        one = cme.Batch([inst], **kw)
+        one.step(1e-2, 3)
+        np.testing.assert_array_equal(together[i], one.get_state())

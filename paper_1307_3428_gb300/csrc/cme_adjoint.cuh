@@ -164,12 +164,9 @@ __global__ void __launch_bounds__(adj_threads<LOGN, R, C>()) segment_kernel(cons
             for (int j = 0; j < R; ++j)
                 sstore(o + j * P, fs.Dh[j]);
         }
-        if constexpr (METHOD == METHOD_RK4IP && C == 1)
-            block_rk4ip_step<true, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c, o,
-                                                                valid ? o + TT : nullptr, TT);
-        else if constexpr (METHOD == METHOD_RK4IP)
-            rk4ip_step_impl<true, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c,
-                                                               valid ? o + TT : nullptr, TT);
+        if constexpr (METHOD == METHOD_RK4IP)
+            rk4ip_step<true, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c, o,
+                                                          valid ? o + TT : nullptr, TT);
         else
             strang_step_impl<true>(grp, fs, pr, c, valid ? o + TT : nullptr, TT);
     }

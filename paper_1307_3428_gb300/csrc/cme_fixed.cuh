@@ -8,14 +8,14 @@
 // such that this bound fits 61 bits, run the passes on integers, and convert back.  The rounding
 // of a pass is then 2^-61 of the bound instead of 2^-53 of each value; against extended precision
 // the transforms are 1.2 to 3 times closer than FP64 ones (N = 4 ... 4096).
-// One radix-8 pass with its twiddles takes 1130 cycles a warp (8 values per thread, one warp per
+// One radix-8 pass with its twiddles takes about 1100 cycles a warp (8 values per thread, one warp per
 // scheduler), where its 84 FP64 instructions per thread took about 6000.
 //
 // Scale.  One reduction per transform gives the largest exponent and L1.  A group of unrelated
-// modes has L1 ~ sqrt(N) times its 2-norm and would leave its values log2(N) bits low; the input
-// is scaled by the bound after the first pass only, min(L1, r |x|max), and the passes shift
-// right where min(L1, L |x|max) grows past 61 bits.  Both bounds are the group's own, powers of
-// two, and independent of the order of the reduction.
+// modes has L1 ~ sqrt(N) times its 2-norm and would leave its values log2(N) bits low; so the scale
+// follows the bounds after every pass, min(L1, (product of the radices so far) |x|max), less the
+// two bits by which each twiddled pass scales down (FixTransform::headroom).  Both bounds are
+// the group's own, powers of two, and independent of the order of the reduction.
 //
 // Multiplication.  A value is x = h 2^32 + l with h and l signed 32-bit ("balanced" limbs: l is
 // the low word read as signed, h the high word plus its carry), so every partial product is a
@@ -74,21 +74,25 @@ CME_DEV long long fshift(long long v, int s)
 {
     return (v + ((1LL << (s - 1)) - 1) + ((v >> s) & 1)) >> s;
 }
-// v 2^-s rounded to nearest, s in 0 ... 63 (uniform over the group)
-CME_DEV long long frsh(long long v, int s) { return s > 0 ? (v + (1LL << (s - 1))) >> s : v; }
-// a (w / 4) 2^-e: twiddled values lose two bits, which the growth of the next pass takes anyway
-CME_DEV fx fcmul4(fx a, fl2 w, int e)
+// the same for s in 0 ... 63 (uniform over the group); EVEN = false rounds ties up, for shifts of
+// many bits or values that only enter a right-hand side
+template <bool EVEN = true>
+CME_DEV long long frsh(long long v, int s)
+{
+    if (s == 0)
+        return v;
+    return EVEN ? fshift(v, s) : (v + (1LL << (s - 1))) >> s;
+}
+// a (w / 4): twiddled values lose two bits, which the growth of the next pass takes anyway
+CME_DEV fx fcmul4(fx a, fl2 w)
 {
     const fl r = fsplit(a.re), i = fsplit(a.im);
     const int nih = -i.h;
     const long long A = fmad(nih, w.im.l, fmad(r.l, w.re.h, fwide(r.h, w.re.l)));
     const long long M = fmad(i.l, w.re.h, fmad(r.l, w.im.h, fwide(r.h, w.im.l)));
     const int t = fhi(A) - fhi(fwide(i.l, w.im.h)), u = fhi(M) - fhi(fwide(nih, w.re.l));
-    fx p = {fmad(t, 1, fmad(nih, w.im.h, fwide(r.h, w.re.h))),
+    return {fmad(t, 1, fmad(nih, w.im.h, fwide(r.h, w.re.h))),
             fmad(u, 1, fmad(i.h, w.re.h, fwide(r.h, w.im.h)))};
-    if (e > 0)   // uniform over the group
-        p = {fshift(p.re, e), fshift(p.im, e)};
-    return p;
 }
 // a w, unscaled (|a| < 2^62)
 CME_DEV fx fcmul1(fx a, fl2 w)
@@ -331,30 +335,36 @@ struct FixTransform {
     static constexpr int KB = LIM - ilog2(PL::radix(0)) < 59 ? LIM - ilog2(PL::radix(0)) : 59;
     using GRd = GroupReduce<P>;
 
-    // extra right shift before pass s >= 1 and the sum of all shifts, from the bounds of the input
-    struct Shifts {
-        int e[NS];
-        int cur;
-    };
-    CME_DEV static Shifts shifts(FixBound b)
+    // Bits that an input of bounds b reaches, over the passes: at most LIM before a run.
+    CME_DEV static int headroom(FixBound b)
     {
-        Shifts h;
-        h.cur = 0;
-        int g = b.bm + ilog2(PL::radix(0));
-        h.e[0] = 0;
+        int g = b.bm + ilog2(PL::radix(0)), h = min(b.bl, g);
 #pragma unroll
         for (int s = 1; s < NS; ++s) {
             g += ilog2(PL::radix(s));
-            h.e[s] = max(0, min(b.bl, g) - LIM - (h.cur + HB));
-            h.cur += HB + h.e[s];
+            h = max(h, min(b.bl, g) - s * HB);
         }
         return h;
     }
+    // the result of a run is X 2^OUT, its modulus in bits
+    static constexpr int OUT = HB * (NS - 1);
+    CME_DEV static int out_bits(FixBound b) { return min(b.bl, b.bm + LOGN) - OUT; }
 
     template <int s, class TW>
-    CME_DEV static void pass(fx (&x)[R], const TW& tw, int e)
+    CME_DEV static void pass(fx (&x)[R], const TW& tw)
     {
         constexpr int r = PL::radix(s), Q = R / r;
+        // Butterflies whose twiddles are all 1 (k = 0; they lead to output 0) floor their products
+        // exactly, without the second floor that cancels the bias elsewhere: each value ends
+        // 3/8 (HB = 1: 1/4) of a unit low.  Their first value is floored too, so that only
+        // output 0 is off, by r times that (`low`), and it is corrected (not where it is 0: zeros
+        // stay zeros).  Without it: output 0 of N = 4096 off by 4 to 12 times the other outputs'
+        // error.
+        constexpr bool fix0 = s > 0 && (HB == 2 || r > 2);
+        constexpr int low = HB == 2 ? (3 * r + 4) / 8 : r / 4;
+        bool k0 = false;
+        if constexpr (fix0)
+            k0 = tw.kst[s] == 0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             fx v[r];
@@ -362,15 +372,22 @@ struct FixTransform {
             for (int j = 0; j < r; ++j)
                 v[j] = x[q + j * Q];
             if constexpr (s > 0) {
-                v[0] = {fshift(v[0].re, HB + e), fshift(v[0].im, HB + e)};
+                constexpr int half = (1 << (HB - 1)) - 1;   // ties to even
+                const bool z = fix0 && k0 && q == 0;
+                const int ar = z ? 0 : half + ((int)(v[0].re >> HB) & 1);
+                const int ai = z ? 0 : half + ((int)(v[0].im >> HB) & 1);
+                v[0] = {(v[0].re + ar) >> HB, (v[0].im + ai) >> HB};
 #pragma unroll
                 for (int j = 1; j < r; ++j) {
                     if constexpr (HB == 1)
                         v[j] = fadd(v[j], v[j]);
-                    v[j] = fcmul4(v[j], tw.template get<s>(q, j), e);
+                    v[j] = fcmul4(v[j], tw.template get<s>(q, j));
                 }
             }
             fdft<r>(v);
+            if (fix0 && q == 0)
+                v[0] = {v[0].re + (k0 && v[0].re != 0 ? low : 0),
+                        v[0].im + (k0 && v[0].im != 0 ? low : 0)};
 #pragma unroll
             for (int j = 0; j < r; ++j)
                 x[q + j * Q] = v[j];
@@ -378,9 +395,9 @@ struct FixTransform {
     }
     template <int s, class TW>
     CME_DEV static void run_from(fx (&x)[R], const TW& tw, const Xbuf<double>& buf, int& par,
-                                 const typename TF::Addr& ad, const Shifts& h)
+                                 const typename TF::Addr& ad)
     {
-        pass<s>(x, tw, h.e[s]);
+        pass<s>(x, tw);
         if constexpr (s + 1 < NS) {
             cx<double> y[R];
 #pragma unroll
@@ -391,14 +408,14 @@ struct FixTransform {
             for (int j = 0; j < R; ++j)
                 x[j] = {__double_as_longlong(y[j].re), __double_as_longlong(y[j].im)};
             par ^= 1;
-            run_from<s + 1>(x, tw, buf, par, ad, h);
+            run_from<s + 1>(x, tw, buf, par, ad);
         }
     }
     template <class TW>
     CME_DEV static void run(fx (&x)[R], const TW& tw, const Xbuf<double>& buf, int& par,
-                            const typename TF::Addr& ad, const Shifts& h)
+                            const typename TF::Addr& ad)
     {
-        run_from<0>(x, tw, buf, par, ad, h);
+        run_from<0>(x, tw, buf, par, ad);
     }
 
     // Scale of a group's FP64 values: X = x 2^q, bounds of X.  q = POISON: a value is not finite.
@@ -440,7 +457,7 @@ struct FixTransform {
         }
         const bool bad = E == 2047;
         const int bl = 32 - __clz((int)cnt) - 12, bm = 2;
-        const int B0 = min(bl, bm + ilog2(PL::radix(0)));
+        const int B0 = headroom({bm, bl});
         const int c0 = 62 - LIM + B0 + E;
 #pragma unroll
         for (int j = 0; j < R; ++j)
@@ -502,7 +519,7 @@ struct FixTransform {
     // are first scaled by their own largest modulus (they lie up to sqrt(N) below the bound of
     // the transform), and L1 of the product comes from the same reduction.
     struct Kerr {
-        int up, us;   // left shifts of the samples and of the products g |a|^2
+        int up, ps, us;   // left shifts of the samples, of |a|^2 and of g |a|^2
         fl G;         // limbs of -g 2^(62 - eg), |g| = m 2^eg with m in [1/2, 1)
         int qc;       // -g |a|^2 is (|a|^2 G) 2^-qc before its shift
         int q;        // scale and bounds of conj(i g |a|^2 a)
@@ -525,10 +542,14 @@ struct FixTransform {
         GRd::template combine<3, 1>(key, cnt, red, t);
         Kerr k;
         k.up = max(61 - 40 - (key >> 1), 0);   // modulus below 2^61
-        // |a|^2 < 2^62, times |g| 2^(62 - eg) < 2^62 and a < 2^61: products below 2^57, and
-        // below 2^KB with the product of |a|^2 and g shifted left by us; an even key leaves
-        // |a|^2 one bit below its bound
-        k.us = KB - 57 + ((key & 1) ^ 1);
+        // |a|^2 < 2^58, shifted left by 4 bits, times |g| 2^(62 - eg) < 2^62 and a < 2^61: products
+        // below 2^57, and below 2^KB with g |a|^2 shifted left by KB - 57; less where the next
+        // transform has no room for that; an even key leaves |a|^2 one bit below its bound
+        const FixBound full = {KB, KB + 32 - __clz((int)cnt) - 12};
+        const int less = max(headroom(full) - LIM, 0);
+        const int sh = KB - 57 - less, odd = (key & 1) ^ 1;
+        k.ps = 4 + min(sh, 0);
+        k.us = max(sh, 0) + odd;
         const int gh = __double2hiint(g);
         const int ge = (gh >> 20) & 0x7ff, eg = ge ? ge - 1022 : 0;
         const long long gm =
@@ -538,9 +559,9 @@ struct FixTransform {
                : 0;
         k.G = fsplit(gh < 0 ? gm : -gm);
         const int qa = q + k.up;
-        k.qc = 2 * qa - 62 - eg;
-        k.q = 3 * qa - 126 + k.us - eg;
-        k.b = {KB, KB + 32 - __clz((int)cnt) - 12};
+        k.qc = 2 * qa - 66 + k.ps - eg;
+        k.q = qa + k.qc + k.us - 64;
+        k.b = {full.bm - less, full.bl - less};
         return k;
     }
     // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc
@@ -548,7 +569,7 @@ struct FixTransform {
     {
         const fl r = fsplit(X.re << k.up), i = fsplit(X.im << k.up);
         const long long m = fmad(i.h, i.l, fmad(r.h, r.l, 0x40000000LL));
-        const long long p2 = fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)) << 4;
+        const long long p2 = fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)) << k.ps;
         const long long pg = fmulhi(fsplit(p2), k.G);
         const fl c = fsplit(pg << k.us);
         X = {fmulhi(c, i), fmulhi(c, r)};
@@ -567,13 +588,15 @@ struct FixTransform {
     // expm1(i phi) = i phi F with the Taylor series F = sin(phi)/phi + i (1 - cos(phi))/phi in
     // phi^2, cut where the group's largest phi leaves less than 2^-62 (5 terms at 0.06); larger
     // phases take sincos in FP64 (no reduction in that branch: groups of a block may differ).
-    // 4 x N = 256 at 4 values per thread: 9.1 -> 5.0 us per split step, most of it the FP64
+    // 4 x N = 256 at 4 values per thread: 9.1 -> 4.8 us per split step, most of it the FP64
     // instructions of sincos (about 3500 cycles per value, against about 350).
+    // LG: log2 of the instance's N (this transform's, or that of its cluster).
+    template <int LG>
     CME_DEV static Kerr kerr_flow(fx (&X)[R], int q, double gh, int2* red, int t)
     {
-        constexpr double invN = 1.0 / N;
+        constexpr double invN = 1.0 / (1 << LG);
         Kerr k = kerr_scale(X, q, gh * invN, red, t);
-        const int sh = k.qc - 62 - LOGN;   // |pg| < 2^60: phi 2^62 = |pg| 2^-sh < 2^(60 - sh)
+        const int sh = k.qc - 62 - LG;   // |pg| < 2^60: phi 2^62 = |pg| 2^-sh < 2^(60 - sh)
         if (sh >= -2) {
             const int terms = sh < 0 ? (sh == -1 ? 8 : 10) : sh < 2 ? 7 : sh < 4 ? 5 : sh < 8 ? 4
                               : sh < 15 ? 3 : 2;
@@ -611,41 +634,48 @@ struct FixTransform {
                 // conj(expm1(i phi)) / 4 as limbs; the product with a, 2^-5 of it
                 const fl2 w = {fsplit(fix(-sn * sn, 1085 - 61)), fsplit(fix(-sn * cs, 1085 - 61))};
                 const fx c = {X[j].re << k.up, -(X[j].im << k.up)};
-                X[j] = fcmul4(c, w, 1);
+                const fx b = fcmul4(c, w);
+                X[j] = {fshift(b.re, 1), fshift(b.im, 1)};
             }
-            k.q = q + k.up - 5 + LOGN;
+            k.q = q + k.up - 5 + LG;
             k.b = {61 - 4, 61 - 4 + LOGN};
+            const int less = max(headroom(k.b) - LIM, 0);
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                X[j] = {frsh(X[j].re, less), frsh(X[j].im, less)};
+            k.q -= less;
+            k.b = {k.b.bm - less, k.b.bl - less};
         }
         return k;
     }
-    // Bounds of values that are below 2^62: the largest component and L1, from their high words.
+    // Bounds of values that are below 2^62.5: the largest component and L1, from their high words.
     CME_DEV static FixBound bounds(const fx (&X)[R], int2* red, int t)
     {
         float mx = 0.f, f = 0.f;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            const float r = fabsf(hi_float(X[j].re)), i = fabsf(hi_float(X[j].im));
+            const float r = fabsf(hi_float<9>(X[j].re)), i = fabsf(hi_float<9>(X[j].im));
             mx = fmaxf(mx, fmaxf(r, i));
             f += r + i;
         }
-        // components below 2^(key + 1) units of 2^40 (each high word is up to 1 below its value)
+        // components below 2^(key + 1) units of 2^41 (each high word is up to 1 below its value)
         int key = (int)(GRd::max_key(__float_as_uint(mx + 1.f)) >> 23) - 127;
         unsigned cnt = GRd::sum(
             (unsigned)((f + 2 * R) * __int_as_float((127 + 11 - key) << 23)) + 1u);
         GRd::template combine<1>(key, cnt, red, t);
-        return {40 + key + 2, 40 + key + 1 + 32 - __clz((int)cnt) - 12};
+        return {41 + key + 2, 41 + key + 1 + 32 - __clz((int)cnt) - 12};
     }
-    // Scale values with bounds b for a transform: right where the first pass could overflow,
+    // Scale values with bounds b for a transform: right where a pass could overflow,
     // left where more than three bits would be lost.  Returns the shift (left positive).
     CME_DEV static int rescale(fx (&X)[R], FixBound& b)
     {
-        const int s = LIM - min(b.bl, b.bm + ilog2(PL::radix(0)));
+        const int s = LIM - headroom(b);
         if (s >= 0 && s <= 3)
             return 0;
         if (s < 0) {
 #pragma unroll
             for (int j = 0; j < R; ++j)
-                X[j] = {frsh(X[j].re, -s), frsh(X[j].im, -s)};
+                X[j] = {frsh<false>(X[j].re, -s), frsh<false>(X[j].im, -s)};
         } else {
 #pragma unroll
             for (int j = 0; j < R; ++j)
@@ -656,23 +686,32 @@ struct FixTransform {
         return s;
     }
     // Common scale of the sum of values v 2^-q, modulus below 2^b, of two sums: the coarser of the
-    // two, and coarse enough that the result's modulus stays below 2^62.
+    // two, and coarse enough that the result's modulus stays below 2^62 (2^62.1 where one is a
+    // sixteenth of the other or less, so that a value at the limit keeps its last bit).
     struct Align {
         int q, sv, sw;   // scale of the sum, right shifts of the two
+        int b;           // bits of the sum
     };
     CME_DEV static Align align(int qv, int bv, int qw, int bw)
     {
         int q = min(qv, qw);
-        q -= max(max(bv - (qv - q), bw - (qw - q)) - 61, 0);
-        return {q, min(qv - q, 63), min(qw - q, 63)};
+        const int cv = bv - (qv - q), cw = bw - (qw - q);
+        const int top = max(cv, cw), sum = top - min(cv, cw) >= 4 ? top : top + 1;
+        const int e = max(sum - 62, 0);
+        q -= e;
+        return {q, min(qv - q, 63), min(qw - q, 63), sum - e};
     }
+    template <bool EVEN>
     CME_DEV static fx asum(fx v, fx w, const Align& a)
     {
-        return {frsh(v.re, a.sv) + frsh(w.re, a.sw), frsh(v.im, a.sv) + frsh(w.im, a.sw)};
+        return {frsh<EVEN>(v.re, a.sv) + frsh<EVEN>(w.re, a.sw),
+                frsh<EVEN>(v.im, a.sv) + frsh<EVEN>(w.im, a.sw)};
     }
+    // v in units of 2^(32 + S), floored; below 2^22 of them
+    template <int S = 8>
     CME_DEV static float hi_float(long long v)
     {
-        return __int_as_float(0x4b400000 + ((int)(v >> 32) >> 8)) - 12582912.f;
+        return __int_as_float(0x4b400000 + ((int)(v >> 32) >> S)) - 12582912.f;
     }
 };
 

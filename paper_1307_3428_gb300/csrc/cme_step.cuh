@@ -133,8 +133,14 @@ struct Group {
     uint32_t rmb[C > 1 ? C : 1];
     uint32_t mb;
     uint32_t om, ot;
-    const cx<T>* twm;
-    const cx<T>* twt;
+    // (FP64: limbs; scw: the source blocks' scale words of receive buffer 0, at byte offset scw_off
+    // of the receive buffers in every block)
+    using TWC = std::conditional_t<sizeof(T) == 8, int4, cx<T>>;
+    const TWC* twm;
+    const TWC* twt;
+    const int2* scw;
+    uint32_t scw_off;
+    int rank;
     int apar;
     uint32_t ph;
     bool timed_out;
@@ -206,15 +212,22 @@ struct Group {
     // reverse order of the stages for a cluster).
     CME_DEV void inverse(cx<T> (&x)[R], int d)
     {
-        if constexpr (C == 1) {
-            block_inverse(x);
+        if constexpr (FIX) {
+            fx X[R];
+            const typename FT::Scale sc = FT::load(x, X, red, tl());
+            int q = sc.q;
+            bool bad = q == FT::POISON;
+            fix_inverse(X, q, sc.b, bad, d);
+            FT::store(X, bad ? -FT::POISON : -q, x);
+        } else if constexpr (C == 1) {
+            TF::template run<+1>(x, tw, buf, par, ad);
         } else {
             if (d == 1) {
                 CF::radix_c(x);
                 twiddle(x, twt);
                 all_to_all<true>(x);
             }
-            block_inverse(x);
+            TF::template run<+1>(x, tw, buf, par, ad);
             if (d == 0) {
                 twiddle(x, twm);
                 all_to_all<false>(x);
@@ -224,20 +237,145 @@ struct Group {
     }
     // this thread's index among those that share a transform's block
     CME_DEV int tl() const { return C == 1 ? t : (int)threadIdx.x; }
-    // the inverse transform inside one block
-    CME_DEV void block_inverse(cx<T> (&x)[R])
+    // The same for fixed-point values X = x 2^q of bounds b; returns the bits of the result's
+    // modulus.  C > 1: every block scales by its own bounds (its modes or samples alone), and
+    // every all-to-all carries each source block's scale word (q, modulus and L1 bits), by
+    // which the receiver aligns that block's values: no reduction over the cluster (16 x N = 4096
+    // on 8-block clusters, RK4IP: 115 us per step in FP64 instructions, see rk4ip_step).
+    CME_DEV int fix_inverse(fx (&X)[R], int& q, FixBound b, bool& bad, int d)
     {
-        if constexpr (FIX) {
-            fx X[R];
-            const typename FT::Scale sc = FT::load(x, X, red, tl());
-            const typename FT::Shifts h = FT::shifts(sc.b);
-            FT::run(X, tw, buf, par, ad, h);
-            FT::store(X, h.cur - sc.q, x);
+        if constexpr (C == 1) {
+            FT::run(X, tw, buf, par, ad);
+            q -= FT::OUT;
+            return FT::out_bits(b);
         } else {
-            TF::template run<+1>(x, tw, buf, par, ad);
+            constexpr int G = CF::G, PC = CF::PC;
+            int bits = 0;
+            int qs[C], bs[C], ls[C];   // the source blocks' scale words
+            if (d == 1) {
+                fix_radix_c(X);
+                // (slots of k1 = 0 have twiddle 1: a rounded shift has no bias, a floored product
+                // by 1 has)
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    X[j] = j < G ? fx{fshift(X[j].re, 2), fshift(X[j].im, 2)}
+                                 : fcmul4(X[j], fl2_of(twt[j * PC]));
+                fix_all_to_all<true>(X, q - 2, min(b.bl, b.bm + LC) - 2, b.bl - 2, bad, qs, bs, ls);
+                q = qs[0];
+#pragma unroll
+                for (int c = 1; c < C; ++c)
+                    q = min(q, qs[c]);
+                // bounds at the coarsest source's scale: every received value is a sum over
+                // all sources' samples of unit-modulus multiples, so L1 is at most the sum of
+                // the sources' L1 (in units of 2^(top - 20))
+                int top = -1000, bm = -1000;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    top = max(top, ls[c] - (qs[c] - q));
+                    bm = max(bm, bs[c] - (qs[c] - q));
+                }
+                unsigned cnt = 0;
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    cnt += (1u << 20) >> min(top - (ls[c] - (qs[c] - q)), 31);
+                b = {bm, top + 32 - __clz((int)(cnt - 1)) - 20};
+                const int s = FT::LIM - FT::headroom(b);
+                const int use = s < 0 || s > 3 ? s : 0;
+                q += use;
+                b.bm += use;
+                b.bl += use;
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    X[j] = align_to(X[j], qs[j % C] - q);
+            }
+            FT::run(X, tw, buf, par, ad);
+            q -= FT::OUT;
+            bits = FT::out_bits(b);
+            if (d == 0) {
+                if (rank != 0) {   // block 0's twiddles are 1
+#pragma unroll
+                    for (int j = 0; j < R; ++j)
+                        X[j] = fcmul4(X[j], fl2_of(twm[j * PC]));
+                    q -= 2;
+                    bits -= 2;
+                }
+                fix_all_to_all<false>(X, q, bits, 0, bad, qs, bs, ls);
+                // a scale at which the C-point sums stay below 2^61
+                q = 1 << 28;
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    q = min(q, qs[c] - max(bs[c] - (61 - LC), 0));
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    X[j] = align_to(X[j], qs[j / G] - q);
+                fix_radix_c(X);
+                bits = 61;
+            }
+            return bits;
         }
     }
-    CME_DEV static void twiddle(cx<T> (&x)[R], const cx<T>* w)
+    CME_DEV static fl2 fl2_of(int4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
+    // v 2^-s, to the left for s < 0 (uniform over the block)
+    CME_DEV static fx align_to(fx v, int s)
+    {
+        if (s < 0)
+            return {v.re << -s, v.im << -s};
+        s = min(s, 63);
+        return {frsh(v.re, s), frsh(v.im, s)};
+    }
+    CME_DEV static void fix_radix_c(fx (&x)[R])
+    {
+        if constexpr (C > 1) {
+#pragma unroll
+            for (int m = 0; m < CF::G; ++m) {
+                fx v[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    v[c] = x[c * CF::G + m];
+                fdft<C>(v);
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    x[c * CF::G + m] = v[c];
+            }
+        }
+    }
+    // all_to_all of fixed-point values with this block's scale word (q, bits of the modulus and of
+    // L1, whether a value was not finite) to every block; qs, bs, ls are the sources'.
+    template <bool T2M>
+    CME_DEV void fix_all_to_all(fx (&X)[R], int q, int bm, int bl, bool& bad, int (&qs)[C],
+                                int (&bs)[C], int (&ls)[C])
+    {
+        cx<double> y[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            y[j] = {__longlong_as_double(X[j].re), __longlong_as_double(X[j].im)};
+        const int buffer = apar;
+        if ((int)threadIdx.x < C && !timed_out) {
+            const int word = ((bm & 0xfff) << 16) | ((bl & 0xfff) << 1) | (bad ? 1 : 0);
+            uint32_t to = 0, tm = 0;
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                if ((int)threadIdx.x == c) {
+                    to = rb[c];
+                    tm = rmb[c];
+                }
+            dsmem_put_async(to + scw_off + (uint32_t)(8 * (buffer * C + rank)),
+                            __hiloint2double(q, word), tm + 8u * (uint32_t)buffer);
+        }
+        all_to_all<T2M>(y);
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            X[j] = {__double_as_longlong(y[j].re), __double_as_longlong(y[j].im)};
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int2 w = scw[buffer * C + c];
+            qs[c] = w.y;
+            bs[c] = (w.x << 4) >> 20;
+            ls[c] = (w.x << 19) >> 20;
+            bad |= (w.x & 1) != 0;
+        }
+    }
+    CME_DEV static void twiddle(cx<T> (&x)[R], const TWC* w)
     {
 #pragma unroll
         for (int j = 0; j < R; ++j)
@@ -268,9 +406,11 @@ struct Group {
                 abuf.put_remote_async(rb[j % C] + om + po + (uint32_t)(8 * PC * (j / C)), x[j],
                                       rmb[j % C] + bo);
         }
-        // the phase ends when this block's one arrival is in and all N2 values have landed
+        // the phase ends when this block's one arrival is in and all N2 values (FP64: and the
+        // C scale words) have landed
         if (threadIdx.x == 0)
-            mbar_arrive_expect_tx(mb + bo, (uint32_t)(CF::N2 * 8 * W + (fault ? 8 : 0)));
+            mbar_arrive_expect_tx(mb + bo, (uint32_t)(CF::N2 * 8 * W + (FIX ? 8 * C : 0) +
+                                                      (fault ? 8 : 0)));
         if (!mbar_wait(mb + bo, (ph >> apar) & 1u, fault ? 1024 : WAIT_TRIES))
             timed_out = true;   // the caller reports the instance
         ph ^= 1u << apar;
@@ -287,7 +427,7 @@ struct Group {
     // The same, also storing the time-domain field a at aout[j P] unless aout is null.
     CME_DEV void rhs_store_a(cx<T> (&x)[R], T gN, cx<T> pump, cx<T>* aout)
     {
-        if constexpr (FIX && C == 1)
+        if constexpr (FIX)
             fix_rhs(x, gN, aout);
         else
             float_rhs(x, gN, aout);
@@ -303,25 +443,25 @@ struct Group {
     {
         fx X[R];
         const typename FT::Scale sc = FT::load(x, X, red, tl());
-        typename FT::Shifts h = FT::shifts(sc.b);
         int q = sc.q;
+        FixBound b = sc.b;
+        bool bad = q == FT::POISON;
 #pragma unroll 1
         for (int d = 0; d < 2; ++d) {
-            FT::run(X, tw, buf, par, ad, h);
-            q -= h.cur;
+            fix_inverse(X, q, b, bad, d);
             if (d == 0) {
                 if (aout) {
-                    FT::store(X, -q, x);
+                    FT::store(X, bad ? -FT::POISON : -q, x);
 #pragma unroll
                     for (int j = 0; j < R; ++j)
                         sstore(aout + j * P, x[j]);
                 }
                 const typename FT::Kerr k = FT::kerr(X, q, gN, red, tl());
                 q = k.q;
-                h = FT::shifts(k.b);
+                b = k.b;
             }
         }
-        FT::store(X, -q, x);
+        FT::store(X, bad ? -FT::POISON : -q, x);
     }
     CME_DEV void float_rhs(cx<T> (&x)[R], T gN, cx<T>* aout)
     {
@@ -384,14 +524,15 @@ struct Group {
     // dynamic shared memory holds the two exchange buffers of its N2-point transform, the two
     // all-to-all receive buffers, the two twiddle arrays of the four-step transform, (FP32,
     // N2 >= 2048) the pass twiddles of the N2-point transform, the receive buffers' two
-    // mbarriers and (FP64) the reduction pairs.
-    CME_DEV void setup_cluster(unsigned char* smem, int rank, int l, const void* tw_table,
+    // mbarriers and (FP64) their scale words and the reduction pairs.
+    CME_DEV void setup_cluster(unsigned char* smem, int rank_, int l, const void* tw_table,
                                int a2a_fault)
     {
         static_assert(C > 1, "cluster groups only");
         constexpr int W = Xbuf<T>::words_per_elem, PC = CF::PC, N2 = CF::N2, G = CF::G;
         unsigned char* a2a = smem + (size_t)2 * TF::BUF * 8 * W;
-        cx<T>* tws = reinterpret_cast<cx<T>*>(a2a + (size_t)2 * N2 * 8 * W);
+        TWC* tws = reinterpret_cast<TWC*>(a2a + (size_t)2 * N2 * 8 * W);
+        rank = rank_;
         if constexpr (sizeof(T) == 4) {
             buf.p = reinterpret_cast<float2*>(smem);
             abuf.p = reinterpret_cast<float2*>(a2a) + l;
@@ -409,7 +550,7 @@ struct Group {
         apar = 0;
         ad = TF::make_addr(l);
         if constexpr (TW_SMEM)
-            tw.init(tw_table, l, tws + 2 * N2);
+            tw.init(tw_table, l, reinterpret_cast<cx<T>*>(tws + 2 * N2));
         else
             tw.init(tw_table, l);
         const uint32_t a0 = smem_addr(a2a);
@@ -420,8 +561,12 @@ struct Group {
             rb[c] = dsmem_map(a0, c);
             rmb[c] = dsmem_map(mb, c);
         }
-        red = reinterpret_cast<int2*>(smem + cluster_smem_bytes<T, LOGN, R, C>() -
-                                      red_bytes(sizeof(T), PC));
+        if constexpr (FIX) {
+            red = reinterpret_cast<int2*>(smem + cluster_smem_bytes<T, LOGN, R, C>() -
+                                          red_bytes(sizeof(T), PC));
+            scw = red - 2 * C;
+            scw_off = smem_addr(scw) - a0;
+        }
         // the kernel's cluster barrier before the first all-to-all publishes the initialisation
         if (l == 0) {
             mbar_init(mb, 1);
@@ -436,12 +581,18 @@ struct Group {
         // exp(2 pi i n2 k1 / N): after the block transform (n2 = l + PC j, k1 = rank), and
         // after the C-point transforms (n2 = rank PC + l + P (i mod G), k1 = i / G)
         const int tp = rank * PC + l;
-        cx<T>* wm = tws + l;
-        cx<T>* wt = tws + N2 + l;
+        TWC* wm = tws + l;
+        TWC* wt = tws + N2 + l;
+        const auto tab = [&](int i) -> TWC {
+            if constexpr (FIX)
+                return __ldg(reinterpret_cast<const int4*>(tw_table) + i);
+            else
+                return gload<T>(tw_table, i);
+        };
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            wm[j * PC] = twload<T>(tw_table, ((l + PC * j) * rank) & (N - 1));
-            wt[j * PC] = twload<T>(tw_table, ((tp + P * (j % G)) * (j / G)) & (N - 1));
+            wm[j * PC] = tab(((l + PC * j) * rank) & (N - 1));
+            wt[j * PC] = tab(((tp + P * (j % G)) * (j / G)) & (N - 1));
         }
         twm = wm;
         twt = wt;
@@ -459,7 +610,7 @@ CME_HD constexpr size_t cluster_smem_bytes()
     return (size_t)2 * CF::TL::BUF * 8 * W + (size_t)2 * CF::N2 * 8 * W +
            (size_t)2 * CF::N2 * sizeof(cx<T>) +
            (Group<T, LOGN, R, C>::TW_SMEM ? tw_bytes(sizeof(T), LOGN - CF::LC, R) : 0) + 16 +
-           red_bytes(sizeof(T), CF::PC);
+           (Group<T, LOGN, R, C>::FIX ? 2 * C * 8 : 0) + red_bytes(sizeof(T), CF::PC);
 }
 
 template <typename T>
@@ -667,7 +818,7 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
     }
 }
 
-// One RK4IP step of an FP64 one-block group with the stages in fixed point (cme_fixed.cuh).  The
+// One RK4IP step of an FP64 group with the stages in fixed point (cme_fixed.cuh).  The
 // state D, its propagation and the step's increment are FP64; what only enters a right-hand side
 // (the stage inputs) or the increment (the right-hand sides and their sum) stays in fixed
 // point, each on its own block scale, as in
@@ -678,21 +829,21 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
 // the same step as rk4ip_step_impl.  Per mode and step that leaves 8 FP64 instructions of the 74
 // outside the transforms, and one conversion from and one to FP64 instead of four each.
 // N = 512 x 256: 88.5 us per step with FP64 instructions throughout (bound by their pipe), 36.8
-// with only the transforms and the Kerr term in fixed point, 23.0 with the stages.  One N = 64
-// instance: 19.5, 11.7 and 7.7 us.  What bounds it now is one warp per scheduler issuing dependent
+// with only the transforms and the Kerr term in fixed point, 21.7 with the stages.  One N = 64
+// instance: 19.5, 11.7 and 7.2 us.  What bounds it now is one warp per scheduler issuing dependent
 // integer instructions (fixed-latency waits, 1.4 per issue).
 // The error of a step against extended precision on the small modes of a comb (1e-6 beside a
-// pumped mode of 1.3, h = 2e-4): 1.3e-21 at N = 512 and 1.4e-21 at 4096, from 4.9e-21 and 1.6e-21
+// pumped mode of 1.3, h = 2e-4): 1.2e-21 at N = 512 and 1.1e-21 at 4096, from 4.9e-21 and 1.6e-21
 // in FP64 instructions.  It is set by the units of the stage inputs and of the increment, so both
 // keep every bit the bounds leave (fcmul1, not fcmul4, there).
 // park: where the state waits in global memory during the step (groups whose registers and shared
 // memory are full: ACC_SMEM), else unused.  STAGES: as in rk4ip_step_impl.
-template <bool STAGES, int LOGN, int R>
-CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, LOGN, R, 1>& fs,
-                            const Props<double, LOGN, R, 1>& pr, const StepConsts<double>& c,
+template <bool STAGES, int LOGN, int R, int C>
+CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, C>& grp, FieldState<double, LOGN, R, C>& fs,
+                            const Props<double, LOGN, R, C>& pr, const StepConsts<double>& c,
                             cx<double>* park, cx<double>* so, long long sstride)
 {
-    using GR = Group<double, LOGN, R, 1>;
+    using GR = Group<double, LOGN, R, C>;
     using FT = typename GR::FT;
     constexpr int P = GR::P;
     constexpr bool AS = GR::ACC_SMEM;
@@ -717,7 +868,7 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, L
         for (int j = 0; j < R; ++j)
             park_store(park + j * P, fs.Dh[j]);
     }
-    const bool bad = sc.q == FT::POISON;
+    bool bad = sc.q == FT::POISON;
     FixBound b = sc.b;
     int q = bad ? 0 : sc.q, bY = 0, qU = q, bU = min(b.bm, b.bl), qA = 0, bA = 0;
 #pragma unroll
@@ -725,16 +876,16 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, L
         U[j] = X[j];
     const double gh = c.gN * c.hh;
     const cx<double> pump = cscale(c.pump, c.hh);
-    // |pump| < 2^eP
-    const int eP = (int)(max(FT::habs(pump.re), FT::habs(pump.im)) >> 20) - 1022 + 1;
+    // |pump| < 2^eP (in the block that holds mode 0)
+    const int eP = C > 1 && grp.rank != 0
+                       ? -4000
+                       : (int)(max(FT::habs(pump.re), FT::habs(pump.im)) >> 20) - 1022 + 1;
 #pragma unroll 1
     for (int st = 0; st < 4; ++st) {
-        typename FT::Shifts h = FT::shifts(b);
         // X becomes Y of this stage, scale q, modulus below 2^bY
 #pragma unroll 1
         for (int d = 0; d < 2; ++d) {
-            FT::run(X, grp.tw, grp.buf, grp.par, grp.ad, h);
-            q -= h.cur;
+            bY = grp.fix_inverse(X, q, b, bad, d);
             if (d == 0) {
                 if constexpr (STAGES) {
                     if (so) {
@@ -748,9 +899,6 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, L
                 const typename FT::Kerr k = FT::kerr(X, q, gh, grp.red, grp.tl());
                 q = k.q - (st == 2);
                 b = k.b;
-                h = FT::shifts(b);
-            } else {
-                bY = min(b.bl, b.bm + LOGN) - h.cur;
             }
         }
         // the sum with the pump stays below 2^62
@@ -792,22 +940,22 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, L
 #pragma unroll
             for (int j = 0; j < R; ++j) {
                 const fl2 E = pr.getF(j);
-                const fx a = fcmul4(X[j], E, 0);
+                const fx a = fcmul4(X[j], E);
                 U[j] = fcmul1(U[j], E);
                 setA(j, a);
-                X[j] = FT::asum(U[j], a, al);
+                X[j] = FT::template asum<false>(U[j], a, al);
             }
             q = al.q;
         } else {
             // A += (2 or 1) Y
             const typename FT::Align aa = FT::align(qA, bA, q - (st == 1), bY);
-            bA = max(bA - (qA - aa.q), bY - (q - (st == 1) - aa.q)) + 1;
+            bA = aa.b;
             qA = aa.q;
             const typename FT::Align al = FT::align(qU, bU, q, bY);
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                setA(j, FT::asum(getA(j), X[j], aa));
-                X[j] = FT::asum(U[j], X[j], al);
+                setA(j, FT::template asum<true>(getA(j), X[j], aa));
+                X[j] = FT::template asum<false>(U[j], X[j], al);
             }
             q = al.q;
             if (st == 2)
@@ -824,7 +972,7 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, 1>& grp, FieldState<double, L
     const typename FT::Align al = FT::align(qA, bA, q, bY);
 #pragma unroll
     for (int j = 0; j < R; ++j)
-        X[j] = FT::asum(fcmul1(getA(j), pr.getF(j)), X[j], al);
+        X[j] = FT::template asum<true>(fcmul1(getA(j), pr.getF(j)), X[j], al);
     cx<double> w[R];
     FT::store(X, bad ? -FT::POISON : -al.q, w);
 #pragma unroll
@@ -845,19 +993,12 @@ CME_HD constexpr bool rk_cache_ed()
     return sizeof(T) == 4 && R <= 8 && Plan<LOGN, R>::P / C <= 256;
 }
 
-template <bool CACHE = false, typename T, int LOGN, int R, int C>
+// The RK4IP step: FP64 in fixed point, except with per-mode Kerr factors (of any size, so without
+// a common scale).
+template <bool STAGES, bool CACHE, typename T, int LOGN, int R, int C>
 CME_DEV void rk4ip_step(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C>& fs,
-                        const Props<T, LOGN, R, C>& pr, const StepConsts<T>& c)
-{
-    rk4ip_step_impl<false, CACHE>(grp, fs, pr, c, static_cast<cx<T>*>(nullptr), 0);
-}
-
-// The RK4IP step of a one-block group: FP64 in fixed point, except with per-mode Kerr factors (of
-// any size, so without a common scale).
-template <bool STAGES, bool CACHE, typename T, int LOGN, int R>
-CME_DEV void block_rk4ip_step(Group<T, LOGN, R, 1>& grp, FieldState<T, LOGN, R, 1>& fs,
-                              const Props<T, LOGN, R, 1>& pr, const StepConsts<T>& c, cx<T>* park,
-                              cx<T>* so, long long sstride)
+                        const Props<T, LOGN, R, C>& pr, const StepConsts<T>& c, cx<T>* park,
+                        cx<T>* so, long long sstride)
 {
     if constexpr (sizeof(T) == 8) {
         if (!grp.km) {
@@ -900,38 +1041,38 @@ CME_DEV void strang_linear(const Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, 
     }
 }
 
-// The same in fixed point (FP64 one-block groups): both transforms, the phase and its exponential.
-template <bool STORE, int LOGN, int R>
-CME_DEV void fix_strang_kerr(Group<double, LOGN, R, 1>& grp, FieldState<double, LOGN, R, 1>& fs,
+// The same in fixed point (FP64): both transforms, the phase and its exponential.
+template <bool STORE, int LOGN, int R, int C>
+CME_DEV void fix_strang_kerr(Group<double, LOGN, R, C>& grp, FieldState<double, LOGN, R, C>& fs,
                              const StepConsts<double>& c, cx<double>* so, long long sstride)
 {
-    using GR = Group<double, LOGN, R, 1>;
+    using GR = Group<double, LOGN, R, C>;
     using FT = typename GR::FT;
     constexpr int P = GR::P;
     fx X[R];
     cx<double> x[R];
     const typename FT::Scale sc = FT::load(fs.Dh, X, grp.red, grp.tl());
-    typename FT::Shifts h = FT::shifts(sc.b);
+    FixBound b = sc.b;
     int q = sc.q;
+    bool bad = q == FT::POISON;
 #pragma unroll 1
     for (int d = 0; d < 2; ++d) {
-        FT::run(X, grp.tw, grp.buf, grp.par, grp.ad, h);
-        q -= h.cur;
+        grp.fix_inverse(X, q, b, bad, d);
         if (d == 0) {
             if constexpr (STORE) {
                 if (so) {
-                    FT::store(X, -q, x);
+                    FT::store(X, bad ? -FT::POISON : -q, x);
 #pragma unroll
                     for (int j = 0; j < R; ++j)
                         sstore(so + j * P, x[j]);
                 }
             }
-            const typename FT::Kerr k = FT::kerr_flow(X, q, 2.0 * c.g0h, grp.red, grp.tl());
+            const typename FT::Kerr k = FT::template kerr_flow<LOGN>(X, q, 2.0 * c.g0h, grp.red, grp.tl());
             q = k.q;
-            h = FT::shifts(k.b);
+            b = k.b;
         }
     }
-    FT::store(X, -q, x);
+    FT::store(X, bad ? -FT::POISON : -q, x);
     grp.mask(x);   // no Kerr increment on padding modes
 #pragma unroll
     for (int j = 0; j < R; ++j)
@@ -953,7 +1094,7 @@ template <bool STORE, typename T, int LOGN, int R, int C>
 CME_DEV void strang_kerr(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C>& fs,
                          const StepConsts<T>& c, cx<T>* so, long long sstride)
 {
-    if constexpr (sizeof(T) == 8 && C == 1) {
+    if constexpr (sizeof(T) == 8) {
         fix_strang_kerr<STORE>(grp, fs, c, so, sstride);
     } else {
     constexpr int P = Group<T, LOGN, R, C>::P;
@@ -1103,7 +1244,7 @@ CME_DEV void step_body(const StepArgs& a, int first, unsigned char* smem)
 
     if constexpr (METHOD == METHOD_RK4IP) {
         for (long long n = 0; n < a.nsteps; ++n)
-            block_rk4ip_step<false, !FUSED && rk_cache_ed<T, LOGN, R, 1>()>(
+            rk4ip_step<false, !FUSED && rk_cache_ed<T, LOGN, R, 1>()>(
                 grp, fs, pr, c, hi, static_cast<cx<T>*>(nullptr), 0);
     } else {
         const long long m = a.single_steps ? 1 : a.nsteps;
@@ -1159,7 +1300,8 @@ __global__ void __launch_bounds__(Plan<LOGN, R>::P / C) cluster_step_kernel(cons
 
     if constexpr (METHOD == METHOD_RK4IP) {
         for (long long n = 0; n < a.nsteps; ++n)
-            rk4ip_step<rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c);
+            rk4ip_step<false, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c, hi,
+                                                            static_cast<cx<T>*>(nullptr), 0);
     } else {
         const long long m = a.single_steps ? 1 : a.nsteps;
         for (long long n = 0; n < a.nsteps; n += m)

@@ -23,6 +23,7 @@
 #include "cme_step.cuh"
 
 namespace cme {
+inline namespace CME_FP32_VARIANT {
 
 template <typename T>
 CME_DEV cx<T> cconj(cx<T> a) { return {a.re, -a.im}; }
@@ -155,26 +156,36 @@ __global__ void __launch_bounds__(adj_threads<LOGN, R, C>()) segment_kernel(cons
     // the two roles, so it is indexed by the coalesced scratch slot ts
     cx<T>* out =
         reinterpret_cast<cx<T>*>(A.stages) + A.slot * A.K * ADJ_VECS * TT + off + grp.ts;
+    const bool keep = valid && A.stages;
     if constexpr (C > 1)
         cluster_sync();   // every block of the cluster runs before the first remote store
     for (long long i = 0; i < ns; ++i) {
         cx<T>* o = out + i * ADJ_VECS * TT;
-        if (valid) {
+        if (keep) {
 #pragma unroll
             for (int j = 0; j < R; ++j)
                 sstore(o + j * P, fs.Dh[j]);
         }
         if constexpr (METHOD == METHOD_RK4IP)
-            rk4ip_step<true, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c, o,
-                                                          valid ? o + TT : nullptr, TT);
+            rk4ip_step<true, rk_cache_ed<T, LOGN, R, C>()>(
+                grp, fs, pr, c, keep ? o : reinterpret_cast<cx<T>*>(A.out_hi) + off + t,
+                keep ? o + TT : nullptr, TT);
         else
-            strang_step_impl<true>(grp, fs, pr, c, valid ? o + TT : nullptr, TT);
+            strang_step_impl<true>(grp, fs, pr, c, keep ? o + TT : nullptr, TT);
     }
     // a gradient whose whole trajectory is stored runs its forward pass through this kernel:
     // the segment's final state starts the next segment (or is the final field)
     if (A.out_hi && valid)
         fs.store(reinterpret_cast<cx<T>*>(A.out_hi) + off + t,
                  reinterpret_cast<cx<T>*>(A.out_lo) + off + t);
+    if (!A.stages) {   // a forward pass alone reports what the step kernels report
+        bool bad = false;
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            bad |= !(isfinite(fs.Dh[j].re) && isfinite(fs.Dh[j].im));
+        if (bad && valid)
+            a.status[inst] = 1;
+    }
     if (grp.failed() && a.status)
         a.status[inst] = 2;
     if constexpr (C > 1)
@@ -533,4 +544,5 @@ __global__ void __launch_bounds__(adj_threads<LOGN, R, C>()) strang_adjoint_kern
         cluster_sync();   // no block leaves while a peer may still address its shared memory
 }
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

@@ -17,7 +17,8 @@ struct AdjArgs {
     void* stages;            // [slots][K][ADJ_VECS][total]: per step of a segment, D,
                              // y1 = F(D), k2, k3, then a = IDFT(stage input) of D, x2, x3, x4
                              // (RK4IP), or D, the time-domain field a of the Kerr flow and the
-                             // state after it (Strang); segment seg uses slot `slot`
+                             // state after it (Strang); segment seg uses slot `slot`; null: the
+                             // recomputation stores nothing (a forward pass alone)
     void* dbar;              // [total] cotangent of the field (carried between launches)
     double2* gL;             // [total] accumulated cotangent of L_mu (re: dL/dRe L, im: dL/dIm L)
     double2* pbar;           // [ninst] cotangent of the pump sqrt(kappa_ext) A_in (RK4IP),

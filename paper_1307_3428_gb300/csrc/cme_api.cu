@@ -943,14 +943,12 @@ StepArgs group_args(cme_batch b, const LaunchGroup& g)
 
 cudaError_t large_steps(cme_batch b, LaunchGroup& g, long long nsteps, cudaStream_t st);
 
-cudaError_t launch_group_step(cme_batch b, LaunchGroup& g, long long nsteps, cudaStream_t st,
-                              bool single_steps = false)
+cudaError_t launch_group_step(cme_batch b, LaunchGroup& g, long long nsteps, cudaStream_t st)
 {
     if (g.large)
         return large_steps(b, g, nsteps, st);
     StepArgs a = group_args(b, g);
     a.nsteps = nsteps;
-    a.single_steps = single_steps;
     // Concurrent groups: the groups whose blocks take over a third of an SM's shared memory
     // anyway launch with all of it, where their blocks fit one per SM together, so that each
     // such block has an SM to itself.  Where two N = 2048 blocks shared an SM, the uneven
@@ -1898,7 +1896,7 @@ extern "C" int cme_grad(cme_batch b, double h, long nsteps, const double* target
         }
     }
     // One launch per group of the recomputation (ADJ_RECOMPUTE) or backward role for segment sg,
-    // its per-step data in slot `slot`; the recomputation starts from checkpoint `ckpt` and,
+    // its per-step data in slot `slot` (-1: not stored); the recomputation starts from checkpoint `ckpt` and,
     // where out_hi is set, leaves its final state there.
     auto run_segment = [&](int role, long long sg, long long slot, long long ckpt, void* out_hi,
                            void* out_lo, cudaStream_t str) -> cudaError_t {
@@ -1912,7 +1910,7 @@ extern "C" int cme_grad(cme_batch b, double h, long nsteps, const double* target
             A.total = b->total;
             A.ckpt_hi = b->g_ckpt_hi;
             A.ckpt_lo = b->g_ckpt_lo ? b->g_ckpt_lo : b->g_ckpt_hi;
-            A.stages = b->g_stages;
+            A.stages = slot >= 0 ? b->g_stages : nullptr;
             A.dbar = b->g_dbar;
             A.gL = b->g_gL;
             A.pbar = b->g_pbar + ga.first;
@@ -1955,10 +1953,9 @@ extern "C" int cme_grad(cme_batch b, double h, long nsteps, const double* target
                 CME_CUDA(cudaMemcpyAsync((char*)b->g_ckpt_lo + s * fb, b->lo, fb,
                                          cudaMemcpyDeviceToDevice, st),
                          "cme_grad: checkpoint");
-            const long long n = std::min(K, (long long)nsteps - s * K);
-            // Strang steps one by one, as the recomputation reproduces them bit for bit
-            for (auto& g : ag)
-                CME_CUDA(launch_group_step(b, g, n, st, true), "cme_grad: forward");
+            // through the recomputation kernel, storing nothing: the recomputation reproduces
+            // its states bit for bit
+            CME_CUDA(run_segment(ADJ_RECOMPUTE, s, -1, s, b->hi, b->lo, st), "cme_grad: forward");
         }
     }
     // loss and its seed

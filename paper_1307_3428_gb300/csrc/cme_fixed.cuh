@@ -25,6 +25,7 @@
 #include "cme_core.cuh"
 
 namespace cme {
+inline namespace CME_FP32_VARIANT {
 
 struct fx {   // fixed-point complex value
     long long re, im;
@@ -715,4 +716,5 @@ struct FixTransform {
     }
 };
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

@@ -6,6 +6,7 @@
 #include "cme_step.cuh"
 
 namespace cme {
+inline namespace CME_FP32_VARIANT {
 
 // Each N's body is a separate (not inlined) function so that it gets its own register
 // allocation instead of sharing one with every other N's body.
@@ -75,4 +76,5 @@ inline cudaError_t launch_fused_t(int method, const FusedArgs& a, int grid, size
     return cudaGetLastError();
 }
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

@@ -6,6 +6,7 @@
 #include "cme_step.cuh"
 
 namespace cme {
+inline namespace CME_FP32_VARIANT {
 
 // Every compiled (log2 N, values per thread) pair.  Values per thread R: 8 is the default;
 // 4 and 16 are alternative launch shapes where they fit in registers without spilling, and 2
@@ -127,4 +128,5 @@ inline cudaError_t launch_diag_shape(const StepArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

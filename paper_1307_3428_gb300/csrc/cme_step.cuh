@@ -8,6 +8,7 @@
 #include "cme_fixed.cuh"
 
 namespace cme {
+inline namespace CME_FP32_VARIANT {
 
 // Threads per block a kernel is compiled for: groups of P >= 64 threads run one instance per
 // block (so the register file is shared by as few threads as possible); narrower groups pack
@@ -735,6 +736,7 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
 {
     constexpr bool COMP = Group<T, LOGN, R, C>::COMP;
     constexpr int P = Group<T, LOGN, R, C>::P;
+    constexpr bool PK = packed_twiddles(LOGN, R);
     cx<T> x[R];
     // CACHE: e1 D (stages 0, 1), then e2 D (stages 2, 3) computed once and kept in registers
     // across the stage's transforms (kernels with registers to spare); else recomputed
@@ -759,9 +761,9 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
 #pragma unroll
             for (int j = 0; j < R; ++j) {
                 const cx<T> E = pr.getE(j);
-                const cx<T> k1 = cmul(E, x[j]);
-                fs.setS(j, cmul(E, k1));
-                const cx<T> e1D = cmul(pr.get1(j), fs.Dh[j]);
+                const cx<T> k1 = cmul_pk<PK>(E, x[j]);
+                fs.setS(j, cmul_pk<PK>(E, k1));
+                const cx<T> e1D = cmul_pk<PK>(pr.get1(j), fs.Dh[j]);
                 if constexpr (CACHE)
                     eD[j] = e1D;
                 x[j] = cadd(fs.Dh[j], caxpy(e1D, c.hh, k1));
@@ -769,20 +771,20 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
         } else if (st == 1) {
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                fs.setS(j, caxpy(fs.getS(j), T(2), cmul(pr.getE(j), x[j])));
+                fs.setS(j, caxpy(fs.getS(j), T(2), cmul_pk<PK>(pr.getE(j), x[j])));
                 cx<T> e1D;
                 if constexpr (CACHE)
                     e1D = eD[j];
                 else
-                    e1D = cmul(pr.get1(j), fs.Dh[j]);
+                    e1D = cmul_pk<PK>(pr.get1(j), fs.Dh[j]);
                 x[j] = cadd(fs.Dh[j], caxpy(e1D, c.hh, x[j]));
             }
         } else if (st == 2) {
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                const cx<T> Ek3 = cmul(pr.getE(j), x[j]);
+                const cx<T> Ek3 = cmul_pk<PK>(pr.getE(j), x[j]);
                 fs.setS(j, caxpy(fs.getS(j), T(2), Ek3));
-                const cx<T> e2D = cmul(pr.get2(j), fs.Dh[j]);
+                const cx<T> e2D = cmul_pk<PK>(pr.get2(j), fs.Dh[j]);
                 if constexpr (CACHE)
                     eD[j] = e2D;
                 x[j] = cadd(fs.Dh[j], caxpy(e2D, c.h, Ek3));
@@ -795,9 +797,9 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
                 if constexpr (CACHE)
                     d = eD[j];
                 else
-                    d = cmul(e2, fs.Dh[j]);
+                    d = cmul_pk<PK>(e2, fs.Dh[j]);
                 if constexpr (COMP)
-                    d = cadd(d, cmul(e2, fs.getL(j)));
+                    d = cadd(d, cmul_pk<PK>(e2, fs.getL(j)));
                 d = caxpy(d, c.h6, cadd(fs.getS(j), x[j]));
                 fs.add(j, d);
             }
@@ -1032,9 +1034,9 @@ CME_DEV void strang_linear(const Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, 
 #pragma unroll
     for (int j = 0; j < R; ++j) {
         const cx<T> e = full ? pr.get2(j) : pr.get1(j);
-        cx<T> d = cmul(e, fs.Dh[j]);
+        cx<T> d = cmul_pk<packed_twiddles(LOGN, R)>(e, fs.Dh[j]);
         if constexpr (COMP)
-            d = cadd(d, cmul(e, fs.getL(j)));
+            d = cadd(d, cmul_pk<packed_twiddles(LOGN, R)>(e, fs.getL(j)));
         if (j == 0 && grp.t == 0)
             d = cadd(d, full ? c.cp2 : c.cp);
         fs.add(j, d);
@@ -1247,9 +1249,7 @@ CME_DEV void step_body(const StepArgs& a, int first, unsigned char* smem)
             rk4ip_step<false, !FUSED && rk_cache_ed<T, LOGN, R, 1>()>(
                 grp, fs, pr, c, hi, static_cast<cx<T>*>(nullptr), 0);
     } else {
-        const long long m = a.single_steps ? 1 : a.nsteps;
-        for (long long n = 0; n < a.nsteps; n += m)
-            strang_steps(grp, fs, pr, c, a.nsteps - n < m ? a.nsteps - n : m);
+        strang_steps(grp, fs, pr, c, a.nsteps);
     }
 
     bool bad = false;
@@ -1303,9 +1303,7 @@ __global__ void __launch_bounds__(Plan<LOGN, R>::P / C) cluster_step_kernel(cons
             rk4ip_step<false, rk_cache_ed<T, LOGN, R, C>()>(grp, fs, pr, c, hi,
                                                             static_cast<cx<T>*>(nullptr), 0);
     } else {
-        const long long m = a.single_steps ? 1 : a.nsteps;
-        for (long long n = 0; n < a.nsteps; n += m)
-            strang_steps(grp, fs, pr, c, a.nsteps - n < m ? a.nsteps - n : m);
+        strang_steps(grp, fs, pr, c, a.nsteps);
     }
 
     bool bad = false;
@@ -1371,4 +1369,5 @@ __global__ void __launch_bounds__(max_threads<LOGN, R>()) diag_kernel(const Step
     }
 }
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

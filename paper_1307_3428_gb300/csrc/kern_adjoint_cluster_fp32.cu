@@ -1,4 +1,5 @@
 // Adjoint kernels of RK4IP, FP32, one instance per thread-block cluster.
+#define CME_FP32_SCALAR   // (cme_core.cuh)
 #include "cme_launch.cuh"
 #include "cme_adjoint.cuh"
 

@@ -1,5 +1,6 @@
 // Adjoint kernels of RK4IP, FP32: per segment, the recomputation of states and stage values
 // and the backward pass.
+#define CME_FP32_SCALAR   // (cme_core.cuh)
 #include "cme_launch.cuh"
 #include "cme_adjoint.cuh"
 

@@ -1,6 +1,7 @@
 // Adjoint kernels of the Strang split step, FP32: per segment, the recomputation of the states
 // and Kerr-flow fields, and the backward pass; one block per instance group or one
 // thread-block cluster per instance.
+#define CME_FP32_SCALAR   // (cme_core.cuh)
 #include "cme_launch.cuh"
 #include "cme_adjoint.cuh"
 

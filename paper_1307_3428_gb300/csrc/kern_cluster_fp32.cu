@@ -1,4 +1,5 @@
 // Cluster step kernels (FP32): one instance per thread-block cluster, both integrators.
+#define CME_FP32_SCALAR   // (cme_core.cuh)
 #include "cme_launch.cuh"
 
 namespace cme {

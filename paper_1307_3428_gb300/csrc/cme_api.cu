@@ -108,7 +108,8 @@ void dev_free(void* p, cme_free_fn f, void* ctx)
 bool shape_compiled(int logN, int R)
 {
     static const int shapes[][2] = {{2, 4},  {3, 8},  {4, 8},  {4, 16}, {5, 8},  {5, 16},
-                                    {6, 8},  {6, 4},  {6, 16}, {6, 2},  {7, 8},  {7, 4},
+                                    {4, 2},  {5, 2},  {6, 8},  {6, 4},  {6, 16},
+                                    {6, 2},  {7, 8},  {7, 4},
                                     {7, 16}, {7, 2},  {8, 8},  {8, 4},  {8, 16}, {9, 8},
                                     {9, 4},  {10, 8}, {10, 4}, {11, 8}, {11, 16}, {12, 8},
                                     {12, 16}};
@@ -121,23 +122,29 @@ bool shape_compiled(int logN, int R)
 // Values per thread: 8 (N = 4: 4), except FP32 N >= 2048, which take 16: with their twiddles
 // in shared memory and their propagators in registers that measured 11.7 against 13.3 us per
 // step at N = 4096 and 7.2 against 7.4 at N = 2048 (GB300).
-// FP64 groups too small to give every SM a warp at 8 values per thread take 4: each thread's
-// chain of FP64 instructions (1/64 of the FP32 rate) then sets the step time, and halving it
-// measured 31 against 55 us per step for one N = 64 instance.  Groups of N = 64 or 128 that
-// hold at most one warp per SM at 2 values per thread take 2, halving the chain again: 19.4
-// against 31 us per step for one N = 64 instance.  sms = 0: no such information.
-int default_radix(int logN, int prec, int count = 0, int sms = 0)
+// FP64 kernels issue long chains of integer instructions per value, so fewer values per thread
+// pay as long as the SMs hold the extra warps side by side: 2 (N <= 128) or 4 (N <= 512, Strang
+// 1024; above, the additional passes cost more) while the group's warps are at most two per
+// scheduler (four schedulers an SM).  RK4IP us per step at 2 / 4 / 8 values, 152 SMs: N = 64 x 1
+// 7.5 / 12.0 / 16.1, x 1216 9.8 / 12.8 / 17.0; N = 128 x 608 11.6 / 12.9 / 19.8, x 1216 (four
+// warps per scheduler at 2, two at 4) 18.6 / 16.2 / 20.0; N = 256 x 608 - / 16.5 / 20.6, x 1216
+// - / 33.1 / 28.1; N = 512 x 256 - / 19.3 / 22.3, x 608 - / 38.6 / 30.0; N = 1024 x 76
+// - / 29.2 / 27.5.  sms = 0: no such information.
+int default_radix(int logN, int prec, int count = 0, int sms = 0, int method = METHOD_RK4IP)
 {
     if (logN <= 2)
         return 4;
     if (prec == PREC_FP32 && logN >= 11)
         return 16;
-    if (prec == PREC_FP64 && sms > 0 && shape_compiled(logN, 2) &&
-        (long long)count * ((1 << logN) / 2) <= 32LL * sms)
-        return 2;
-    if (prec == PREC_FP64 && sms > 0 && shape_compiled(logN, 4) &&
-        (long long)count * ((1 << logN) / 8) < 32LL * sms)
-        return 4;
+    if (prec == PREC_FP64 && sms > 0) {
+        const int most[2] = {7, method == METHOD_STRANG ? 10 : 9};   // log2 N at 2 and at 4 values
+        for (int i = 0; i < 2; ++i) {
+            const int r = 2 << i;
+            const long long warps = ((long long)count * ((1 << logN) / r) + 31) / 32;
+            if (logN <= most[i] && shape_compiled(logN, r) && warps <= 8LL * sms)
+                return r;
+        }
+    }
     return 8;
 }
 
@@ -285,6 +292,30 @@ int inst_per_block(int N, int R, int G, int count)
     return std::min(G, count);
 }
 
+// Clusters for groups of N = 2048 and 4096 whose one-block plan leaves SMs idle: the largest C
+// that `allowed(group, C)` and whose blocks, with the other groups', stay within ~3.4 per SM.
+template <typename F>
+void choose_clusters(std::vector<LaunchGroup>& groups, int sms, F allowed)
+{
+    long long blocks1 = 0;
+    for (const auto& g : groups)
+        blocks1 += (g.count + g.G - 1) / g.G;
+    const long long cap = (long long)sms * 17 / 5;
+    if (3 * blocks1 > 2LL * sms)
+        return;
+    for (auto& g : groups) {
+        const long long others = blocks1 - (g.count + g.G - 1) / g.G;
+        for (int c : {8, 4, 2})
+            if ((g.logN == 11 || g.logN == 12) && cluster_shape_compiled(g.logN, 8, c) &&
+                allowed(g, c) && others + (long long)g.count * c <= cap) {
+                g.C = c;
+                g.R = 8;
+                g.G = 1;
+                break;
+            }
+    }
+}
+
 // (Re)compute the launch plan of every group from the options: values per thread R and
 // instances per block G of the per-group kernels, and the persistent work-list tiles.
 int plan_batch(cme_batch b, const cme_options& o)
@@ -314,14 +345,15 @@ int plan_batch(cme_batch b, const cme_options& o)
             any_large = true;
             continue;
         }
-        int R = o.radix ? o.radix : default_radix(g.logN, b->prec, g.count, b->sms);
+        int R = o.radix ? o.radix : default_radix(g.logN, b->prec, g.count, b->sms, b->method);
         // an explicit cluster request without an explicit radix takes the clusters' 8 values
         // per thread
         if (!o.radix && o.cluster > 1 && cluster_shape_compiled(g.logN, 8, o.cluster))
             R = 8;
         if (R > g.N)
             R = g.N;
-        if (!shape_compiled(g.logN, R))
+        // (2 values per thread on request at N = 64, 128 only)
+        if (!shape_compiled(g.logN, R) || (o.radix == 2 && g.logN != 6 && g.logN != 7))
             return fail(CME_ERR_INVALID_ARG, "launch plan: radix %d not available for N=%d", R, g.N);
         g.R = R;
         g.G = inst_per_block(g.N, R, o.inst_per_cta, g.count);
@@ -332,36 +364,21 @@ int plan_batch(cme_batch b, const cme_options& o)
     }
     // Library choice of clusters (o.cluster == 0).  Only where one block per instance leaves
     // SMs idle: the batch's one-block plan occupies at most 2/3 of the SMs.  A group of
-    // N = 2048 or 4096 then takes the largest cluster whose blocks, with the other groups',
-    // stay within ~3.4 per SM (all resident at once), at 8 values per thread: C = 8 in FP32
-    // (C = 4 and 2 lose to one block there), C = 8, 4 or 2 in FP64.  Measured per RK4IP step,
+    // N = 2048 (FP32) or 4096 then takes 8-block clusters if its blocks, with the other groups',
+    // stay within ~3.4 per SM (all resident at once), at 8 values per thread; smaller clusters
+    // lose to one block.  Measured per RK4IP step,
     // FP32 N = 4096: 16 instances 11.5 -> 5.9 us, 64 instances 11.7 -> 8.2 us, 96 instances
-    // 11.7 -> 15.5 us (not all blocks resident); FP64 N = 4096: 16 instances 437 -> 115 us,
-    // 96 instances 437 -> 349 us (C = 4).  Mixed batches whose one-block plan fills the GPU
+    // 11.7 -> 15.5 us (not all blocks resident); FP64 N = 4096: 16 instances 108 -> 65 us, 64
+    // instances 108 -> 74 us, 100 instances 109 -> 146 us (C = 4: 166); FP64 N = 2048: 16
+    // instances 52 -> 59 us.  Mixed batches whose one-block plan fills the GPU
     // (N = 256 ... 4096 x 64) keep one block per instance: 584 ms per run, against 776 ms with
     // 8-block clusters.
-    if (o.cluster == 0 && !any_large && o.persistent != 2) {   // the work-list kernel has no clusters
-        long long blocks1 = 0;
-        for (const auto& g : b->groups)
-            blocks1 += (g.count + g.G - 1) / g.G;
-        const long long cap = (long long)b->sms * 17 / 5;
-        if (3 * blocks1 <= 2LL * b->sms) {
-            for (auto& g : b->groups) {
-                if (!(g.logN == 11 || g.logN == 12) || (o.radix && o.radix != 8))
-                    continue;
-                const long long others = blocks1 - (g.count + g.G - 1) / g.G;
-                for (int c : {8, 4, 2}) {
-                    if (b->prec == PREC_FP32 && c < 8)
-                        break;
-                    if (cluster_shape_compiled(g.logN, 8, c) && others + (long long)g.count * c <= cap) {
-                        g.C = c;
-                        g.R = 8;
-                        g.G = 1;
-                        break;
-                    }
-                }
-            }
-        }
+    if (o.cluster == 0 && !any_large && o.persistent != 2 &&   // the work-list kernel has no clusters
+        (o.radix == 0 || o.radix == 8)) {
+        const int first = b->prec == PREC_FP32 ? 11 : 12;
+        choose_clusters(b->groups, b->sms, [&](const LaunchGroup& g, int c) {
+            return g.logN >= first && c == 8;
+        });
     }
     // library choice: one kernel per N group on concurrent streams (measured ahead of the
     // work-list kernel on the uneven N = 256 ... 4096 workload: 1.13 s against 1.22 s)
@@ -1871,8 +1888,13 @@ extern "C" int cme_grad(cme_batch b, double h, long nsteps, const double* target
     // size, FP32 groups of N = 2048, 4096 take the largest cluster for which the
     // recomputation and the backward kernel, which run side by side, both get their own SMs
     // (N = 4096 x 16: 47.2 us per gradient step on one block, 28.5 on 4-block clusters,
-    // 46.2 on 8-block clusters sharing SMs).  FP64 keeps the batch's plan.
+    // 46.2 on 8-block clusters sharing SMs).  FP64 keeps the batch's plan, except that the
+    // backward pass, bound by FP64 instructions, spreads N = 2048 and 4096 over the largest
+    // cluster that fits, also where the forward pass alone runs faster on one block.
     std::vector<LaunchGroup> ag(b->groups);
+    if (b->prec == PREC_FP64 && b->opt.cluster == 0 && b->opt.persistent != 2 &&
+        (b->opt.radix == 0 || b->opt.radix == 8))
+        choose_clusters(ag, b->sms, [](const LaunchGroup& g, int) { return g.C == 1; });
     for (auto& g : ag) {
         g.chunk = nullptr;   // copies never own the chunk graphs
         if (b->prec != PREC_FP32 || g.large)

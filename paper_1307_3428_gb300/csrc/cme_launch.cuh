@@ -14,8 +14,8 @@ inline namespace CME_FP32_VARIANT {
 #define CME_FOR_EACH_SHAPE(X)          \
     X(2, 4)                            \
     X(3, 8)                            \
-    X(4, 8) X(4, 16)                   \
-    X(5, 8) X(5, 16)                   \
+    X(4, 8) X(4, 16) X(4, 2)           \
+    X(5, 8) X(5, 16) X(5, 2)           \
     X(6, 8) X(6, 4) X(6, 16) X(6, 2)   \
     X(7, 8) X(7, 4) X(7, 16) X(7, 2)   \
     X(8, 8) X(8, 4) X(8, 16)           \

@@ -147,3 +147,23 @@ def test_split_step_phases_of_one_block_scale_apart():
         one = cme.Batch([inst], **kw)
         one.step(1e-2, 3)
         np.testing.assert_array_equal(together[i], one.get_state())
+
+
+def test_fp64_plan_by_group_size():
+    """Values per thread of FP64 groups: 2 (N <= 128) and 4 (N <= 512) while their warps are at most
+    two per scheduler, then more; one block per instance at N = 2048; 2 values only on request at
+    N = 64 and 128."""
+    torch = pytest.importorskip("torch")
+    room = 8 * torch.cuda.get_device_properties(0).multi_processor_count   # warps
+    inst = {N: cme.Instance(N, np.ones(N), np.zeros(N), 1.0, 0.5, 0.7, 1.0, np.zeros(N, complex))
+            for N in (16, 32, 64, 128, 256, 512, 1024, 2048)}
+    for N, count, radix in ((16, 1, 2), (16, 4 * room, 2), (16, 4 * room + 1, 8), (32, 2 * room, 2),
+                            (64, room, 2), (64, room + 1, 4), (128, room // 2, 2),
+                            (128, room // 2 + 1, 4), (128, room + 1, 8), (256, room // 2, 4),
+                            (256, room // 2 + 1, 8), (512, room // 4, 4), (512, room // 4 + 1, 8),
+                            (1024, 1, 8), (2048, 1, 8)):
+        b = cme.Batch([inst[N]] * count)
+        assert (b.plan(0)["radix"], b.plan(0)["cluster"]) == (radix, 1), (N, count, b.plan(0))
+        b.close()
+    with pytest.raises(cme.CmeError):
+        cme.Batch([inst[16]], radix=2)

@@ -45,7 +45,8 @@ extern "C" {
 #define CME_ERR_STATE (-7)         /* call out of order (e.g. instance without a field) */
 
 /* ---- options ----------------------------------------------------------------------- */
-#define CME_FP64 0 /* FP64 field, transforms, Kerr term and propagators */
+#define CME_FP64 0 /* FP64 field and propagators; transforms, Kerr term and RK4IP stages to FP64
+                      accuracy, computed in 64-bit fixed point with one scale per instance */
 #define CME_FP32 1 /* FP32 field, transforms and Kerr term; propagators computed in FP64 and
                       applied as small increments; state kept as a compensated FP32 pair */
 
@@ -89,10 +90,10 @@ typedef struct cme_options {
                               0 = library choice: clusters only where one block per
                               instance would leave SMs idle (the batch's one-block plan uses
                               at most 2/3 of them) and not with persistent = 2; a group of
-                              N = 2048 or 4096 then takes the largest C whose blocks, with
-                              the other groups', stay within ~3.4 per SM: C = 8 in FP32
-                              (smaller FP32 clusters do not repay their all-to-all), C = 8,
-                              4 or 2 in FP64.  FP32 gradients take the largest C in {8, 4}
+                              N = 2048 (FP32) or 4096 then takes C = 8 if its blocks, with
+                              the other groups', stay within ~3.4 per SM (smaller clusters do
+                              not repay their all-to-all).  FP64 gradients take the largest C
+                              that fits for both sizes; FP32 gradients take the largest C in {8, 4}
                               with 2 * instances * C <= SMs, since their recomputation and
                               backward kernels run side by side.  Groups without a compiled
                               cluster shape run C = 1. */

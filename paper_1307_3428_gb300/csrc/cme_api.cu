@@ -119,6 +119,9 @@ bool shape_compiled(int logN, int R)
     return false;
 }
 
+// The shapes a caller may name: 2 values per thread at N = 16 and 32 are the library's choice only.
+bool radix_on_request(int logN, int R) { return shape_compiled(logN, R) && (R != 2 || logN >= 6); }
+
 // Values per thread: 8 (N = 4: 4), except FP32 N >= 2048, which take 16: with their twiddles
 // in shared memory and their propagators in registers that measured 11.7 against 13.3 us per
 // step at N = 4096 and 7.2 against 7.4 at N = 2048 (GB300).
@@ -352,8 +355,7 @@ int plan_batch(cme_batch b, const cme_options& o)
             R = 8;
         if (R > g.N)
             R = g.N;
-        // (2 values per thread on request at N = 64, 128 only)
-        if (!shape_compiled(g.logN, R) || (o.radix == 2 && g.logN != 6 && g.logN != 7))
+        if (!(o.radix ? radix_on_request(g.logN, R) : shape_compiled(g.logN, R)))
             return fail(CME_ERR_INVALID_ARG, "launch plan: radix %d not available for N=%d", R, g.N);
         g.R = R;
         g.G = inst_per_block(g.N, R, o.inst_per_cta, g.count);
@@ -681,7 +683,7 @@ int cme_batch_create(const cme_instance* v, int count, const cme_options* opt, v
             continue;
         }
         const int R = std::min(o.radix ? o.radix : default_radix(g.logN, b->prec), N);
-        if (!shape_compiled(g.logN, R) || o.persistent < 0 || o.persistent > 2 ||
+        if (!radix_on_request(g.logN, R) || o.persistent < 0 || o.persistent > 2 ||
             !(o.cluster == 0 || o.cluster == 1 || o.cluster == 2 || o.cluster == 4 ||
               o.cluster == 8)) {
             cme_batch_destroy(b);
@@ -1394,6 +1396,16 @@ int cme_autotune(cme_batch b, double h, long probe_steps, cme_options* plan_out)
         for (int R : {2, 4, 8, 16}) {
             if (R > g.N || !shape_compiled(g.logN, R))
                 continue;
+            if (!radix_on_request(g.logN, R)) {   // reachable as the library's choice, or not at all
+                cme_options o = base;
+                o.radix = 0;
+                o.inst_per_cta = 0;
+                o.persistent = 1;
+                o.cluster = 1;
+                if (default_radix(g.logN, b->prec, g.count, b->sms, b->method) == R)
+                    cand.push_back(o);
+                continue;
+            }
             for (int G : {0, 2, 4}) {
                 const int P = g.N / R;
                 if (G && (P >= 64 || G * P > 256))

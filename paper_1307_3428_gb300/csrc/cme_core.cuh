@@ -20,10 +20,11 @@
 #define CME_HD __host__ __device__
 
 // FP32 arithmetic comes in two variants, one per translation unit: packed (add, mul and fma on
-// (re, im) pairs, half the issue slots) for the one-block step and the four-step kernels, scalar
-// (CME_FP32_SCALAR) for the gradient's kernels and the clusters.  The two round in different
-// orders; a gradient's forward pass, recomputation and backward pass have to be of one, and the
-// clusters, bound by the latency of their all-to-alls, lose 1 to 6% with the packed one.
+// (re, im) pairs, half the issue slots) for the one-block step and the four-step kernels of 2^15 to
+// 2^18 modes, scalar (CME_FP32_SCALAR) for the other four-step kernels, the gradient's kernels and
+// the clusters.  The two round in different orders; a gradient's forward pass, recomputation and
+// backward pass have to be of one, and the clusters, bound by the latency of their all-to-alls,
+// lose 1 to 6% with the packed one.
 #ifdef CME_FP32_SCALAR
 #define CME_FP32_PACKED 0
 #define CME_FP32_VARIANT fp32_scalar

@@ -236,12 +236,16 @@ struct LargeArgs;
 cudaError_t launch_large_row_fp32(int logN2, int R, const LargeArgs& a, long long rows,
                                   cudaStream_t s,
                                   bool pdl);
+cudaError_t launch_large_row_fp32_scalar(int logN2, int R, const LargeArgs& a, long long rows,
+                                         cudaStream_t s, bool pdl);
 cudaError_t launch_large_row_fp64(int logN2, int R, const LargeArgs& a, long long rows,
                                   cudaStream_t s,
                                   bool pdl);
 cudaError_t launch_large_col_fp32(int logN1, int R, const LargeArgs& a, long long cols,
                                   cudaStream_t s,
                                   bool pdl);
+cudaError_t launch_large_col_fp32_scalar(int logN1, int R, const LargeArgs& a, long long cols,
+                                         cudaStream_t s, bool pdl);
 cudaError_t launch_large_col_fp64(int logN1, int R, const LargeArgs& a, long long cols,
                                   cudaStream_t s,
                                   bool pdl);

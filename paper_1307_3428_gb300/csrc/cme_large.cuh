@@ -63,6 +63,8 @@ struct LargeArgs {
     int bar_fault;           // test of the bounded waits: every barrier expects one arrival more
 };
 
+inline namespace CME_FP32_VARIANT {
+
 // Programmatic dependent launch: the step's kernels are launched so that each may start while
 // its predecessor finishes.  A kernel reads only constant data (propagators, twiddles) before
 // pdl_wait(), which returns once the predecessor has completed and its writes are visible; every
@@ -551,4 +553,5 @@ __global__ void __launch_bounds__(Plan<LOGN1, R>::P) large_grid_kernel(const Lar
         A.status[ci] = 2;
 }
 
+}  // namespace CME_FP32_VARIANT
 }  // namespace cme

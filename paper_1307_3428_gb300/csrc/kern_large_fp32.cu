@@ -1,25 +1,31 @@
-// Large-N (four-step) row and column kernels, FP32.
-#include "cme_launch.cuh"
-#include "cme_large.cuh"
+// Large-N (four-step) row and column kernels, FP32: packed arithmetic, and the choice.
+#include "cme_large_launch.cuh"
 
 namespace cme {
 
-#define CME_LARGE_SHAPES(X) \
-    X(6, 8) X(7, 8) X(8, 8) X(9, 8) X(10, 8) X(8, 4) X(9, 4) X(10, 4)
+#define CME_LARGE_ROWS(X) X(7, 8) X(8, 8) X(9, 8) X(8, 4) X(9, 4)
+#define CME_LARGE_COLS(X) X(8, 8) X(9, 8) X(8, 4) X(9, 4)
+
+// Packed arithmetic for 2^15 <= N <= 2^18, scalar (kern_large_fp32_scalar.cu) for the others.
+// us per step, scalar / packed: 2^13 17.2 / 17.8, 8 instances 20.5 / 23.7; 2^14 18.5 / 18.7;
+// 2^15 20.5 / 20.2; 2^16 28.5 / 28.1; 2^17 29.8 / 29.4; 2^18 x 3 114.6 / 114.2; 2^19 98.6 / 102.4;
+// 2^20 152.1 / 154.0 (columns of N1 = 1024: 178 registers, two blocks per SM where 164 leave three).
+static bool packed(const LargeArgs& a)
+{
+    const int logN = a.logN1 + a.logN2;
+    return logN >= 15 && logN <= 18;
+}
 
 cudaError_t launch_large_row_fp32(int logN2, int R, const LargeArgs& a, long long rows,
-                                  cudaStream_t s,
-                                  bool pdl)
+                                  cudaStream_t s, bool pdl)
 {
+    if (!packed(a))
+        return launch_large_row_fp32_scalar(logN2, R, a, rows, s, pdl);
     switch (logN2 * 32 + R) {
-#define CME_CASE(LN, RR)                                                          \
-    case LN * 32 + RR: {                                                                    \
-        constexpr int P = Plan<LN, RR>::P;                                        \
-        const size_t smem = smem_bytes_for<float>(LN, RR, a.G);                    \
-        auto k = large_row_kernel<float, LN, RR>;                                  \
-        return launch_pdl(k, (unsigned)((rows + a.G - 1) / a.G), P * a.G, smem, s, pdl, a); \
-    }
-        CME_LARGE_SHAPES(CME_CASE)
+#define CME_CASE(LN, RR)                                                                    \
+    case LN * 32 + RR:                                                                      \
+        return large_row_launch<float, LN, RR>(a, rows, s, pdl);
+        CME_LARGE_ROWS(CME_CASE)
 #undef CME_CASE
     default:
         return cudaErrorInvalidValue;
@@ -27,39 +33,15 @@ cudaError_t launch_large_row_fp32(int logN2, int R, const LargeArgs& a, long lon
 }
 
 cudaError_t launch_large_col_fp32(int logN1, int R, const LargeArgs& a, long long cols,
-                                  cudaStream_t s,
-                                  bool pdl)
+                                  cudaStream_t s, bool pdl)
 {
+    if (!packed(a))
+        return launch_large_col_fp32_scalar(logN1, R, a, cols, s, pdl);
     switch (logN1 * 32 + R) {
-#define CME_CASE(LN, RR)                                                          \
-    case LN * 32 + RR: {                                                                    \
-        constexpr int P = Plan<LN, RR>::P;                                        \
-        const size_t smem = smem_bytes_for<float>(LN, RR, a.G);                    \
-        const unsigned blocks = (unsigned)((cols + a.G - 1) / a.G);                \
-        switch (a.stage) {                                                         \
-        case LARGE_START:                                                          \
-            return launch_pdl(large_col_kernel<float, LN, RR, LARGE_START>, blocks, P * a.G, \
-                              smem, s, pdl, a);                                    \
-        case 0:                                                                    \
-            return launch_pdl(large_col_kernel<float, LN, RR, 0>, blocks, P * a.G, smem, s, \
-                              pdl, a);                                             \
-        case 1:                                                                    \
-            return launch_pdl(large_col_kernel<float, LN, RR, 1>, blocks, P * a.G, smem, s, \
-                              pdl, a);                                             \
-        case 2:                                                                    \
-            return launch_pdl(large_col_kernel<float, LN, RR, 2>, blocks, P * a.G, smem, s, \
-                              pdl, a);                                             \
-        case 3:                                                                    \
-            return launch_pdl(large_col_kernel<float, LN, RR, 3>, blocks, P * a.G, smem, s, \
-                              pdl, a);                                             \
-        case LARGE_FINAL:                                                          \
-            return launch_pdl(large_col_kernel<float, LN, RR, LARGE_FINAL>, blocks, P * a.G, \
-                              smem, s, pdl, a);                                    \
-        default:                                                                   \
-            return cudaErrorInvalidValue;                                          \
-        }                                                                          \
-    }
-        CME_LARGE_SHAPES(CME_CASE)
+#define CME_CASE(LN, RR)                                                                    \
+    case LN * 32 + RR:                                                                      \
+        return large_col_launch<float, LN, RR>(a, cols, s, pdl);
+        CME_LARGE_COLS(CME_CASE)
 #undef CME_CASE
     default:
         return cudaErrorInvalidValue;

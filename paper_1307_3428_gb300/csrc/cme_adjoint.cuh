@@ -192,81 +192,6 @@ __global__ void __launch_bounds__(adj_threads<LOGN, R, C>()) segment_kernel(cons
         cluster_sync();   // no block leaves while a peer may still address its shared memory
 }
 
-// acc + a conj(b)
-CME_DEV cx<double> cmaccc(cx<double> acc, cx<double> a, cx<double> b)
-{
-    return {fma(a.re, b.re, fma(a.im, b.im, acc.re)), fma(a.im, b.re, fma(-a.re, b.im, acc.im))};
-}
-// The reverse of one RK4IP step in FP64 (adjoint_kernel has the formulas): the vector-Jacobian
-// products in fixed point, the cotangents themselves (whose sizes differ by many decades between
-// modes) in FP64.  The three terms of the L cotangent share the factor conj(h/2 E), which is
-// applied once to their sum: 88 FP64 instructions per mode and step, from 182.
-// 16 x N = 4096 on 8-block clusters: 111 -> 95 us per backward step.
-template <typename LD, int LOGN, int R, int C>
-CME_DEV void adjoint_step_f64(Group<double, LOGN, R, C>& grp, const Props<double, LOGN, R, C>& pr,
-                              const StepConsts<double>& c, const LD& ld, cx<double> (&Db)[R],
-                              LAcc<double> (&gl)[R], LAcc<double>& pb)
-{
-    using cd = cx<double>;
-    const double h = c.h, hh = c.hh, h6 = c.h6, h3 = 2.0 * c.h6;
-    cd ub[R], cot[R], S[R];   // S: conj(w) Dbar' + conj(v) x4bar + conj(D) ubar + conj(y1) k1bar
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const cd E = pr.getE(j);
-        const cd w = caxpy(caxpy(cmul(E, ld(0, j)), h3, cadd(ld(2, j), ld(3, j))), h6,
-                           cmul(E, ld(1, j)));
-        cot[j] = cscale(Db[j], h6);
-        S[j] = cmulc(Db[j], w);
-    }
-#pragma unroll 1
-    for (int st = 3; st >= 0; --st) {
-        if (grp.t == 0)
-            pb.add(cot[0]);
-        cd z[R];
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-            z[j] = cot[j];
-        grp.out_modes(z);
-        grp.fix_vjp(z, c.gN, [&](int j) { return ld(4 + st, j); });
-        grp.mask(z);
-        // z holds conj(stage-input cotangent)
-        if (st == 0) {
-#pragma unroll
-            for (int j = 0; j < R; ++j)
-                Db[j] = cadd(Db[j], cconj(z[j]));
-        } else if (st == 3) {
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const cd xb = cconj(z[j]), E = pr.getE(j);
-                const cd wb = cmulc(Db[j], E), vb = cmulc(xb, E);
-                S[j] = cmaccc(S[j], xb, caxpy(cmul(E, ld(0, j)), h, ld(3, j)));
-                ub[j] = cadd(wb, vb);
-                cot[j] = caxpy(cscale(wb, h3), h, vb);
-            }
-        } else if (st == 2) {
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const cd xb = cconj(z[j]);
-                const cd wb = cmulc(Db[j], pr.getE(j));
-                ub[j] = cadd(ub[j], xb);
-                cot[j] = caxpy(cscale(wb, h3), hh, xb);
-            }
-        } else {   // st == 1
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const cd xb = cconj(z[j]), E = pr.getE(j);
-                const cd wb = cmulc(Db[j], E);
-                ub[j] = cadd(ub[j], xb);
-                const cd k1b = caxpy(cscale(wb, h6), hh, xb);
-                const cd s = cmaccc(cmaccc(S[j], ub[j], ld(0, j)), k1b, ld(1, j));
-                gl[j].add(cscale(cmulc(s, E), hh));
-                Db[j] = cmulc(ub[j], E);
-                cot[j] = cmulc(k1b, E);
-            }
-        }
-    }
-}
-
 // Backward role: the discrete adjoint of the steps of segment A.seg, last step first, from
 // the states, stage values and stage fields in half (A.seg mod 2) of A.stages.  The field cotangent, the
 // L cotangents and the pump cotangent are carried between segments in A.dbar, A.gL, A.pbar.
@@ -364,10 +289,6 @@ __global__ void __launch_bounds__(adj_threads<LOGN, R, C>()) adjoint_kernel(cons
             else
                 return Dn[(long long)v * TT + j * P];
         };
-        if constexpr (sizeof(T) == 8) {
-            adjoint_step_f64(grp, pr, c, ld, Db, gl, pb);
-            continue;
-        }
         // reverse stages 3 (x4), 2 (x3), 1 (x2), 0 (D)
         cx<T> ub[R], cot[R];
 #pragma unroll 1

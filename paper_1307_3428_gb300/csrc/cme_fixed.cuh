@@ -1,15 +1,15 @@
 // FP64 transforms in 64-bit fixed point.
 //
 // FP64 instructions run at 1/64 of the FP32 rate on this GPU: a DADD or DFMA holds its scheduler
-// for 64 to 76 cycles, where a 64-bit integer add takes 3 and a 32 x 32 -> 64 multiply about 4
-// (one warp per scheduler).  A transform only adds, subtracts and rotates, and every
+// for 64 to 76 cycles, where a 64-bit integer add takes 3 and a 32 x 32 -> 64 multiply 2 (one
+// warp per scheduler).  A transform only adds, subtracts and rotates, and every
 // intermediate value is a partial sum of unit-modulus multiples of its inputs, so its modulus is
 // at most L1 = sum |x_k|.  The FP64 kernels therefore scale a group's values by one power of two
-// such that this bound fits 62 bits, run the passes on integers, and convert back.  The rounding
-// of a pass is then 2^-62 of the bound instead of 2^-53 of each value; against extended precision
+// such that this bound fits 61 bits, run the passes on integers, and convert back.  The rounding
+// of a pass is then 2^-61 of the bound instead of 2^-53 of each value; against extended precision
 // the transforms are 1.2 to 3 times closer than FP64 ones (N = 4 ... 4096).
-// One radix-8 pass with its twiddles takes about 1100 cycles a warp (8 values per thread, one
-// warp per scheduler), where its 84 FP64 instructions per thread took about 6000.
+// One radix-8 pass with its twiddles takes about 1100 cycles a warp (8 values per thread, one warp per
+// scheduler), where its 84 FP64 instructions per thread took about 6000.
 //
 // Scale.  One reduction per transform gives the largest exponent and L1.  A group of unrelated
 // modes has L1 ~ sqrt(N) times its 2-norm and would leave its values log2(N) bits low; so the scale
@@ -427,9 +427,7 @@ struct FixTransform {
     };
     CME_DEV static unsigned habs(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
-    // FP64 -> fixed point.  `red`: the group's reduction pairs (P > 32).  TRANSFORM = false: values
-    // that are only multiplied, moduli below 2^62 whatever their sum (no bounds returned).
-    template <bool TRANSFORM = true>
+    // FP64 -> fixed point.  `red`: the group's reduction pairs (P > 32).
     CME_DEV static Scale load(const cx<double> (&xin)[R], fx (&X)[R], int2* red, int t)
     {
         cx<double> x[R];
@@ -440,18 +438,15 @@ struct FixTransform {
             mh = max(mh, max(habs(x[j].re), habs(x[j].im)));
         }
         int E = (int)(GRd::max_key(mh) >> 20);   // biased exponent (the warp's)
-        unsigned cnt = 0;
-        if constexpr (TRANSFORM) {
-            // sum of |re| + |im| in units of 2^(E - 1023), from the leading 20 bits of each
-            const int base = (E - 127) * (1 << 20);
-            float f = 0.f;
+        // sum of |re| + |im| in units of 2^(E - 1023), from the leading 20 bits of each
+        const int base = (E - 127) * (1 << 20);
+        float f = 0.f;
 #pragma unroll
-            for (int j = 0; j < R; ++j) {
-                f += __int_as_float(max((int)habs(x[j].re) - base, 0) << 3);
-                f += __int_as_float(max((int)habs(x[j].im) - base, 0) << 3);
-            }
-            cnt = GRd::sum((unsigned)(f * 4096.f) + 1u);
+        for (int j = 0; j < R; ++j) {
+            f += __int_as_float(max((int)habs(x[j].re) - base, 0) << 3);
+            f += __int_as_float(max((int)habs(x[j].im) - base, 0) << 3);
         }
+        unsigned cnt = GRd::sum((unsigned)(f * 4096.f) + 1u);
         GRd::template combine<1>(E, cnt, red, t);
         int pre = 0;
         if (E < 100) {   // near the denormal range (or all zero): scale up first
@@ -463,7 +458,7 @@ struct FixTransform {
         }
         const bool bad = E == 2047;
         const int bl = 32 - __clz((int)cnt) - 12, bm = 2;
-        const int B0 = TRANSFORM ? headroom({bm, bl}) : bm + LIM - 62;
+        const int B0 = headroom({bm, bl});
         const int c0 = 62 - LIM + B0 + E;
 #pragma unroll
         for (int j = 0; j < R; ++j)
@@ -556,26 +551,19 @@ struct FixTransform {
         const int sh = KB - 57 - less, odd = (key & 1) ^ 1;
         k.ps = 4 + min(sh, 0);
         k.us = max(sh, 0) + odd;
-        int eg;
-        const long long gm = mantissa(g, eg);
-        k.G = fsplit(-gm);
-        const int qa = q + k.up;
-        k.qc = 2 * qa - 66 + k.ps - eg;
-        k.q = qa + k.qc + k.us - 64;
-        k.b = {full.bm - less, full.bl - less};
-        return k;
-    }
-    // g 2^(62 - eg) with |g| = m 2^eg, m in [1/2, 1)
-    CME_DEV static long long mantissa(double g, int& eg)
-    {
-        const int gh = __double2hiint(g), ge = (gh >> 20) & 0x7ff;
-        eg = ge ? ge - 1022 : 0;
+        const int gh = __double2hiint(g);
+        const int ge = (gh >> 20) & 0x7ff, eg = ge ? ge - 1022 : 0;
         const long long gm =
             ge ? (long long)((((unsigned long long)((gh & 0xfffff) | 0x100000) << 32) |
                               (unsigned)__double2loint(g))
                              << 9)
                : 0;
-        return gh < 0 ? -gm : gm;
+        k.G = fsplit(gh < 0 ? gm : -gm);
+        const int qa = q + k.up;
+        k.qc = 2 * qa - 66 + k.ps - eg;
+        k.q = qa + k.qc + k.us - 64;
+        k.b = {full.bm - less, full.bl - less};
+        return k;
     }
     // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc
     CME_DEV static long long kerr_term(fx& X, const Kerr& k)
@@ -660,43 +648,6 @@ struct FixTransform {
             k.b = {k.b.bm - less, k.b.bl - less};
         }
         return k;
-    }
-    // Vector-Jacobian product of the Kerr term at the samples a 2^qa, for the cotangent B 2^q (one
-    // IDFT of the output cotangent): X = B becomes conj(2 |a|^2 b + a^2 conj(b)), b = -i g B, for the
-    // next transform, with its scale q and bounds.  The three coefficients 3 re^2 + im^2,
-    // re^2 + 3 im^2 and 2 re im carry g.  Components of A below 2^61 and of B below 2^61.5, both
-    // close to it: |a|^2 < 2^59, coefficients below 2^60.6 and then 2^62.6, products below 2^61.
-    CME_DEV static void vjp(fx (&X)[R], int& q, FixBound& b, const fx (&A)[R], int qa, double g,
-                            int2* red, int t)
-    {
-        int eg;
-        const fl G = fsplit(mantissa(g, eg));
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const fl r = fsplit(A[j].re), i = fsplit(A[j].im);
-            const long long rr = fmulhi(r, r), ii = fmulhi(i, i), ri = fmulhi(r, i);
-            const fl v = fsplit(fmulhi(fsplit((rr * 3 + ii) << 2), G) << 2);
-            const fl u = fsplit(fmulhi(fsplit((rr + ii * 3) << 2), G) << 2);
-            const fl w = fsplit(fmulhi(fsplit(ri << 3), G) << 2);
-            const fl br = fsplit(X[j].re), bi = fsplit(X[j].im);
-            X[j] = {fmulhi(v, bi) - fmulhi(w, br), fmulhi(u, br) - fmulhi(w, bi)};
-        }
-        q += 2 * qa - 126 - eg;
-        b = bounds(X, red, t);
-        q += rescale(X, b);
-    }
-    // scale values to components in 2^60 ... 2^61 (the largest)
-    CME_DEV static int normalise(fx (&X)[R], int2* red, int t)
-    {
-        const int s = 62 - bounds(X, red, t).bm;
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            if (s >= 0)
-                X[j] = {X[j].re << s, X[j].im << s};
-            else
-                X[j] = {frsh(X[j].re, -s), frsh(X[j].im, -s)};
-        }
-        return s;
     }
     // Bounds of values that are below 2^62.5: the largest component and L1, from their high words.
     CME_DEV static FixBound bounds(const fx (&X)[R], int2* red, int t)

@@ -72,11 +72,11 @@ __host__ __device__ constexpr size_t tw_bytes(int tbytes, int logN, int R)
                      ((1 << logN) / R) * 8
                : 0;
 }
-// FP64 groups wider than a warp: two sets of one (key, count) pair per warp for the scales of the
-// fixed-point transforms
+// FP64 groups wider than a warp: one (key, count) pair per warp for the scale of the fixed-point
+// transforms
 __host__ __device__ constexpr size_t red_bytes(int tbytes, int P)
 {
-    return tbytes == 8 && P > 32 ? (size_t)(P / 32) * 16 : 0;
+    return tbytes == 8 && P > 32 ? (size_t)(P / 32) * 8 : 0;
 }
 __host__ __device__ constexpr size_t group_smem_bytes(int tbytes, int logN, int R)
 {

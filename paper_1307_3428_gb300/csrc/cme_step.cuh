@@ -315,30 +315,6 @@ struct Group {
             return bits;
         }
     }
-    // FP64: z = conj(VJP of the right-hand side's Kerr part at the time samples a) for the output
-    // cotangent z: two transforms and the product in fixed point.  The reductions alternate
-    // between the two sets of pairs where no transform (and so no barrier) lies between them.
-    template <class LD>
-    CME_DEV void fix_vjp(cx<T> (&z)[R], T g, const LD& a)
-    {
-        fx X[R], A[R];
-        const typename FT::Scale sc = FT::load(z, X, red, tl());
-        int q = sc.q;
-        FixBound b = sc.b;
-        bool bad = q == FT::POISON;
-        fix_inverse(X, q, b, bad, 0);
-        q += FT::normalise(X, red, tl());
-        cx<T> av[R];
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-            av[j] = a(j);
-        const typename FT::Scale sa =
-            FT::template load<false>(av, A, red + FT::GRd::W, tl());
-        bad |= sa.q == FT::POISON;
-        FT::vjp(X, q, b, A, sa.q, g, red, tl());
-        fix_inverse(X, q, b, bad, 1);
-        FT::store(X, bad ? -FT::POISON : -q, z);
-    }
     CME_DEV static fl2 fl2_of(int4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
     // v 2^-s, to the left for s < 0 (uniform over the block)
     CME_DEV static fx align_to(fx v, int s)

@@ -167,6 +167,7 @@ CME_DEV void store(void* p, long long i, cx<T> a)
 }
 // A value that waits in global memory (this thread's own slot) and is read back by the same
 // thread; volatile, so that it does not stay in registers instead.
+#ifndef CME_HOST_PRIMITIVES
 CME_DEV void park_store(cx<double>* p, cx<double> v)
 {
     asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.re), "d"(v.im) : "memory");
@@ -177,6 +178,7 @@ CME_DEV cx<double> park_load(const cx<double>* p)
     asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "l"(p) : "memory");
     return v;
 }
+#endif
 
 // ----------------------------------------------------------------------------------------
 // Transform plan: N = 2^LOGN, R values per thread, NS passes, last radix 2^LOG_LAST.

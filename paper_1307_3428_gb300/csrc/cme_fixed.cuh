@@ -42,7 +42,8 @@ CME_DEV fl fsplit(long long v)
     const unsigned lo = (unsigned)v;
     return {(int)((unsigned)(v >> 32) + (lo >> 31)), (int)lo};
 }
-// a b and a b + c
+// a b, a b + c and v 2^s
+#ifndef CME_HOST_PRIMITIVES   // (a host build supplies these, with overflow checks)
 CME_DEV long long fwide(int a, int b)
 {
     long long d;
@@ -55,6 +56,8 @@ CME_DEV long long fmad(int a, int b, long long c)
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
+CME_DEV long long fshl(long long v, int s) { return (long long)((unsigned long long)v << s); }
+#endif
 CME_DEV int fhi(long long v) { return (int)(v >> 32); }
 
 // Products.  The middle sum (h l' + l h') 2^-32 is taken as the difference of two floors, whose
@@ -106,7 +109,7 @@ CME_DEV fx fcmul1(fx a, fl2 w)
         i.l, w.re.h, fmad(i.h, w.re.l, fmad(r.l, w.im.h, fmad(r.h, w.im.l, half))));
     const long long hr = fmad(nih, w.im.h, fwide(r.h, w.re.h));
     const long long hi = fmad(i.h, w.re.h, fwide(r.h, w.im.h));
-    return {(hr << 2) + ((A - fwide(i.l, w.im.h)) >> 30), (hi << 2) + (M >> 30)};
+    return {fshl(hr, 2) + ((A - fwide(i.l, w.im.h)) >> 30), fshl(hi, 2) + (M >> 30)};
 }
 CME_DEV fx fadd(fx a, fx b) { return {a.re + b.re, a.im + b.im}; }
 CME_DEV fx fsub(fx a, fx b) { return {a.re - b.re, a.im - b.im}; }
@@ -329,14 +332,21 @@ struct FixTransform {
     // inputs are doubled first, so that 7 passes cost 7 bits and not 14.
     static constexpr int HB = R <= 4 ? 1 : 2;
     // Bits of every value's modulus: sqrt(2) 2^62 is the largest sum inside a rotation, and the
-    // middle products of fcmul4 stay below 2^63.  Samples reach the Kerr term below 2^61: with a
-    // single pass, which scales nothing, that is the limit.
+    // middle products of fcmul4 stay below 2^63.  With a single pass, which scales nothing, and with
+    // narrow ones 61, the limit of samples that the Kerr term takes (SAMPLE).
+    static constexpr int SAMPLE = 61;
     static constexpr int LIM = HB == 1 || NS == 1 ? 61 : 62;
     // modulus of a product of the Kerr term: room for the first pass's growth (59: its limbs')
     static constexpr int KB = LIM - ilog2(PL::radix(0)) < 59 ? LIM - ilog2(PL::radix(0)) : 59;
     using GRd = GroupReduce<P>;
 
-    // Bits that an input of bounds b reaches, over the passes: at most LIM before a run.
+    static constexpr int OUT = HB * (NS - 1);   // the result of a run is X 2^OUT
+
+    // Bits that an input of bounds b reaches, over the passes: at most LIM before a run.  KERR: the
+    // result goes to the Kerr term, so that it counts LIM - SAMPLE bits more than the passes.  (Where
+    // the last pass is the largest, on short pulses with their flat spectra, it left samples of up
+    // to 2^62, and the Kerr term overflowed: error of order 1.  Other fields keep their scale.)
+    template <bool KERR>
     CME_DEV static int headroom(FixBound b)
     {
         int g = b.bm + ilog2(PL::radix(0)), h = min(b.bl, g);
@@ -345,10 +355,11 @@ struct FixTransform {
             g += ilog2(PL::radix(s));
             h = max(h, min(b.bl, g) - s * HB);
         }
+        if constexpr (KERR && LIM > SAMPLE)
+            h = max(h, min(b.bl, g) - OUT + (LIM - SAMPLE));
         return h;
     }
-    // the result of a run is X 2^OUT, its modulus in bits
-    static constexpr int OUT = HB * (NS - 1);
+    // bits of the result's modulus
     CME_DEV static int out_bits(FixBound b) { return min(b.bl, b.bm + LOGN) - OUT; }
 
     template <int s, class TW>
@@ -427,7 +438,8 @@ struct FixTransform {
     };
     CME_DEV static unsigned habs(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
-    // FP64 -> fixed point.  `red`: the group's reduction pairs (P > 32).
+    // FP64 -> fixed point.  `red`: the group's reduction pairs (P > 32).  KERR: see headroom.
+    template <bool KERR>
     CME_DEV static Scale load(const cx<double> (&xin)[R], fx (&X)[R], int2* red, int t)
     {
         cx<double> x[R];
@@ -458,7 +470,7 @@ struct FixTransform {
         }
         const bool bad = E == 2047;
         const int bl = 32 - __clz((int)cnt) - 12, bm = 2;
-        const int B0 = headroom({bm, bl});
+        const int B0 = headroom<KERR>({bm, bl});
         const int c0 = 62 - LIM + B0 + E;
 #pragma unroll
         for (int j = 0; j < R; ++j)
@@ -492,7 +504,7 @@ struct FixTransform {
             e -= 32;
         }
         const int z = __clz((int)h);
-        const unsigned mh = __funnelshift_l(l, h, z), ml = l << z;
+        const unsigned mh = __funnelshift_l(l, h, z), ml = __funnelshift_l(0u, l, z);
         const unsigned long long d =
             ((((unsigned long long)((mh >> 11) + ((unsigned)(e - z) << 20))) << 32) |
              __funnelshift_r(ml, mh, 11)) +
@@ -516,9 +528,9 @@ struct FixTransform {
         }
     }
 
-    // Scales of the Kerr term of the time samples a = X 2^-q with the coefficient g.  The samples
-    // are first scaled by their own largest modulus (they lie up to sqrt(N) below the bound of
-    // the transform), and L1 of the product comes from the same reduction.
+    // Scales of the Kerr term of the time samples a = X 2^-q, |X| <= 2^SAMPLE, with the coefficient g.
+    // The samples are first scaled by their own largest modulus (they lie up to sqrt(N) below the
+    // bound of the transform), and L1 of the product comes from the same reduction.
     struct Kerr {
         int up, ps, us;   // left shifts of the samples, of |a|^2 and of g |a|^2
         fl G;         // limbs of -g 2^(62 - eg), |g| = m 2^eg with m in [1/2, 1)
@@ -536,18 +548,22 @@ struct FixTransform {
             mx = fmaxf(mx, p);
             f += p * (fabsf(r) + fabsf(i));
         }
-        // |a|^2 below 2^(key - 1), the modulus below 2^hb, units of 2^40
-        int key = max((int)(GRd::max_key(__float_as_uint(mx * 1.02f)) >> 23) - 127 + 2, 2);
+        // |a|^2 below 2^(key - 1), the modulus below 2^(key / 2), units of 2^40.  A component lies up
+        // to one unit above its floor: |a|^2 < p + 2 sqrt(2 p) + 2 <= 1.02 p + 102.  The samples'
+        // limit of 2^21 units gives key = 43, also where 1.02 p exceeds its square.
+        int key = min((int)(GRd::max_key(__float_as_uint(fmaf(mx, 1.02f, 102.f))) >> 23) - 127 + 2,
+                      2 * (SAMPLE - 40) + 1);
         unsigned cnt = GRd::sum(
             (unsigned)(f * __int_as_float((127 + 12 - 3 * (key >> 1)) << 23)) + 1u);
         GRd::template combine<3, 1>(key, cnt, red, t);
         Kerr k;
-        k.up = max(61 - 40 - (key >> 1), 0);   // modulus below 2^61
-        // |a|^2 < 2^58, shifted left by 4 bits, times |g| 2^(62 - eg) < 2^62 and a < 2^61: products
-        // below 2^57, and below 2^KB with g |a|^2 shifted left by KB - 57; less where the next
-        // transform has no room for that; an even key leaves |a|^2 one bit below its bound
+        k.up = SAMPLE - 40 - (key >> 1);   // modulus below 2^61
+        // |a|^2 2^-64 <= 2^58, shifted left by 4 bits, times |g| 2^(62 - eg) < 2^62 and a <= 2^61:
+        // products below 2^57, and below 2^KB with g |a|^2 <= 2^60 shifted left by KB - 57 <= 2;
+        // less where the next transform has no room for that; an even key leaves |a|^2 one bit
+        // below its bound, so that the shift is one more
         const FixBound full = {KB, KB + 32 - __clz((int)cnt) - 12};
-        const int less = max(headroom(full) - LIM, 0);
+        const int less = max(headroom<false>(full) - LIM, 0);
         const int sh = KB - 57 - less, odd = (key & 1) ^ 1;
         k.ps = 4 + min(sh, 0);
         k.us = max(sh, 0) + odd;
@@ -568,11 +584,11 @@ struct FixTransform {
     // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc
     CME_DEV static long long kerr_term(fx& X, const Kerr& k)
     {
-        const fl r = fsplit(X.re << k.up), i = fsplit(X.im << k.up);
+        const fl r = fsplit(fshl(X.re, k.up)), i = fsplit(fshl(X.im, k.up));
         const long long m = fmad(i.h, i.l, fmad(r.h, r.l, 0x40000000LL));
-        const long long p2 = fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)) << k.ps;
+        const long long p2 = fshl(fmad(i.h, i.h, fmad(r.h, r.h, m >> 31)), k.ps);
         const long long pg = fmulhi(fsplit(p2), k.G);
-        const fl c = fsplit(pg << k.us);
+        const fl c = fsplit(fshl(pg, k.us));
         X = {fmulhi(c, i), fmulhi(c, r)};
         return pg;
     }
@@ -607,9 +623,9 @@ struct FixTransform {
             fl z[R];
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                ph[j] = ((-kerr_term(X[j], k)) << ls) >> rs;
+                ph[j] = fshl(-kerr_term(X[j], k), ls) >> rs;
                 const fl p = fsplit(ph[j]);
-                z[j] = fsplit(fmulhi(p, p) << 2);
+                z[j] = fsplit(fshl(fmulhi(p, p), 2));
                 S[j] = {0, 0};
             }
 #pragma unroll 1
@@ -617,12 +633,12 @@ struct FixTransform {
                 const long long cs = fx_sinc[n], cc = fx_cosc[n];
 #pragma unroll
                 for (int j = 0; j < R; ++j)
-                    S[j] = {cs + (fmulhi(fsplit(S[j].re), z[j]) << 2),
-                            cc + (fmulhi(fsplit(S[j].im), z[j]) << 2)};
+                    S[j] = {cs + fshl(fmulhi(fsplit(S[j].re), z[j]), 2),
+                            cc + fshl(fmulhi(fsplit(S[j].im), z[j]), 2)};
             }
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                const long long im = fmulhi(fsplit(S[j].im), fsplit(ph[j])) << 2;
+                const long long im = fshl(fmulhi(fsplit(S[j].im), fsplit(ph[j])), 2);
                 X[j] = fcmul1(X[j], {fsplit(S[j].re), fsplit(-im)});
             }
         } else {
@@ -634,13 +650,13 @@ struct FixTransform {
                 sincos(0.5 * gh * (a[j].re * a[j].re + a[j].im * a[j].im), &sn, &cs);
                 // conj(expm1(i phi)) / 4 as limbs; the product with a, 2^-5 of it
                 const fl2 w = {fsplit(fix(-sn * sn, 1085 - 61)), fsplit(fix(-sn * cs, 1085 - 61))};
-                const fx c = {X[j].re << k.up, -(X[j].im << k.up)};
+                const fx c = {fshl(X[j].re, k.up), -fshl(X[j].im, k.up)};
                 const fx b = fcmul4(c, w);
                 X[j] = {fshift(b.re, 1), fshift(b.im, 1)};
             }
             k.q = q + k.up - 5 + LG;
             k.b = {61 - 4, 61 - 4 + LOGN};
-            const int less = max(headroom(k.b) - LIM, 0);
+            const int less = max(headroom<false>(k.b) - LIM, 0);
 #pragma unroll
             for (int j = 0; j < R; ++j)
                 X[j] = {frsh(X[j].re, less), frsh(X[j].im, less)};
@@ -668,9 +684,10 @@ struct FixTransform {
     }
     // Scale values with bounds b for a transform: right where a pass could overflow,
     // left where more than three bits would be lost.  Returns the shift (left positive).
+    template <bool KERR>
     CME_DEV static int rescale(fx (&X)[R], FixBound& b)
     {
-        const int s = LIM - headroom(b);
+        const int s = LIM - headroom<KERR>(b);
         if (s >= 0 && s <= 3)
             return 0;
         if (s < 0) {
@@ -680,7 +697,7 @@ struct FixTransform {
         } else {
 #pragma unroll
             for (int j = 0; j < R; ++j)
-                X[j] = {X[j].re << s, X[j].im << s};
+                X[j] = {fshl(X[j].re, s), fshl(X[j].im, s)};
         }
         b.bm += s;
         b.bl += s;

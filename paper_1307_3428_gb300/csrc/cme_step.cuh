@@ -115,6 +115,9 @@ struct Group {
         FIX, FixTwiddles<LOGN - LC, R, TW_REGS, C>,
         std::conditional_t<TW_SMEM, TwiddlesSmem<T, LOGN - LC, R, C>,
                            Twiddles<T, LOGN - LC, R, TW_REGS, C>>>;
+    // the block's own transform leaves the Kerr term's samples (a cluster's radix-C sums follow it,
+    // whose scale is chosen for them)
+    static constexpr bool TO_KERR = C == 1;
     int2* red;     // FP64: reduction pairs of this group's warps (shared memory)
 
     int t;         // the thread holds modes t + jP
@@ -215,7 +218,7 @@ struct Group {
     {
         if constexpr (FIX) {
             fx X[R];
-            const typename FT::Scale sc = FT::load(x, X, red, tl());
+            const typename FT::Scale sc = FT::template load<false>(x, X, red, tl());
             int q = sc.q;
             bool bad = q == FT::POISON;
             fix_inverse(X, q, sc.b, bad, d);
@@ -280,7 +283,7 @@ struct Group {
                 for (int c = 0; c < C; ++c)
                     cnt += (1u << 20) >> min(top - (ls[c] - (qs[c] - q)), 31);
                 b = {bm, top + 32 - __clz((int)(cnt - 1)) - 20};
-                const int s = FT::LIM - FT::headroom(b);
+                const int s = FT::LIM - FT::template headroom<false>(b);
                 const int use = s < 0 || s > 3 ? s : 0;
                 q += use;
                 b.bm += use;
@@ -320,7 +323,7 @@ struct Group {
     CME_DEV static fx align_to(fx v, int s)
     {
         if (s < 0)
-            return {v.re << -s, v.im << -s};
+            return {fshl(v.re, -s), fshl(v.im, -s)};
         s = min(s, 63);
         return {frsh(v.re, s), frsh(v.im, s)};
     }
@@ -443,7 +446,7 @@ struct Group {
     CME_DEV void fix_rhs(cx<T> (&x)[R], T gN, cx<T>* aout)
     {
         fx X[R];
-        const typename FT::Scale sc = FT::load(x, X, red, tl());
+        const typename FT::Scale sc = FT::template load<TO_KERR>(x, X, red, tl());
         int q = sc.q;
         FixBound b = sc.b;
         bool bad = q == FT::POISON;
@@ -864,7 +867,7 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, C>& grp, FieldState<double, L
         else
             Ar[j] = v;
     };
-    const typename FT::Scale sc = FT::load(fs.Dh, X, grp.red, grp.tl());
+    const typename FT::Scale sc = FT::template load<GR::TO_KERR>(fs.Dh, X, grp.red, grp.tl());
     if constexpr (AS) {
 #pragma unroll
         for (int j = 0; j < R; ++j)
@@ -966,7 +969,7 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, C>& grp, FieldState<double, L
                     X[j] = fcmul1(X[j], pr.getF(j));
         }
         b = FT::bounds(X, grp.red, grp.tl());
-        q += FT::rescale(X, b);
+        q += FT::template rescale<GR::TO_KERR>(X, b);
     }
     // the increment (E A + Y4) / 3
     // (unscaled product: the increment's unit, relative to its largest mode, is what limits the
@@ -1053,7 +1056,7 @@ CME_DEV void fix_strang_kerr(Group<double, LOGN, R, C>& grp, FieldState<double, 
     constexpr int P = GR::P;
     fx X[R];
     cx<double> x[R];
-    const typename FT::Scale sc = FT::load(fs.Dh, X, grp.red, grp.tl());
+    const typename FT::Scale sc = FT::template load<GR::TO_KERR>(fs.Dh, X, grp.red, grp.tl());
     FixBound b = sc.b;
     int q = sc.q;
     bool bad = q == FT::POISON;

@@ -1,0 +1,132 @@
+"""The FP64 steps' 64-bit fixed point (csrc/cme_fixed.cuh) on the CPU: the device source itself, built
+for the host with overflow checks on every signed sum, product and shift, for every compiled launch
+shape, against extended precision.
+
+The fields are those that reach a bound: a spectrum of equal modes is one sample in time, the
+largest sample that a transform can leave, and a sech spectrum is a pulse; sixteen mantissas over
+one octave move the largest value from just above a power of two to just below the next.
+
+Bounds: an FP64 transform rounds every value once per level, a relative 2-norm error of 2^-53
+per level.  The Kerr term triples the relative error of the samples, and in these fields the samples
+that carry the term carry the 2-norm too; so the right-hand side gets 4 x (levels + 2) roundings.  A
+step adds one right-hand side (the split step's Kerr flow, the weighted sum of the four stages) and
+rounds each mode a few times: 8 x (levels + 4), as in test_gpu_fixed.py."""
+import concurrent.futures as cf
+import os
+import re
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1307_3428_gb300", "csrc")
+L = np.clongdouble
+ULP = 2.0 ** -53
+G0, KAPPA, SIGMA = 1.3, 1.0, 1.0
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+
+
+def shapes():
+    text = open(os.path.join(CSRC, "cme_launch.cuh")).read()
+    macro = re.search(r"#define CME_FOR_EACH_SHAPE\(X\)(.*?[^\\])\n", text, re.S).group(1)
+    return [(int(a), int(b)) for a, b in re.findall(r"X\((\d+), (\d+)\)", macro)]
+
+
+def host_build(out, logN, R):
+    exe = str(out / f"fixed_{logN}_{R}")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-g1", "-ffp-contract=off",
+                    "-fsanitize=signed-integer-overflow,shift", "-fno-sanitize-recover=all",
+                    "-I", os.path.join(ROOT, "tests", "host_fixed"), "-I", CSRC,
+                    "-I", os.path.join(ROOT, "include"), f"-DCASE_LOGN={logN}", f"-DCASE_R={R}",
+                    os.path.join(ROOT, "tests", "host_fixed", "fixed.cpp"), "-o", exe],
+                   check=True, capture_output=True)
+    return exe
+
+
+@pytest.fixture(scope="module")
+def builds(tmp_path_factory):
+    out = tmp_path_factory.mktemp("fixed")
+    with cf.ThreadPoolExecutor(os.cpu_count()) as pool:
+        made = pool.map(lambda s: host_build(out, *s), shapes())
+        return dict(zip(shapes(), made))
+
+
+def run(exe, what, fields, tmp_path, g0=G0, pump=0.0, h=1e-3, steps=1):
+    """`fields` [n, N] (transform order) after the right-hand side or `steps` steps."""
+    src, dst = tmp_path / "in", tmp_path / "out"
+    np.ascontiguousarray(fields, complex).tofile(src)
+    r = subprocess.run([exe, what, *(repr(float(v)) for v in (g0, KAPPA, pump, h)), str(steps), src, dst],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[:400]
+    return np.fromfile(dst, complex).reshape(fields.shape)
+
+
+def pulses(N):
+    """Spectra of short pulses: equal modes (real, imaginary, at 45 degrees, at a time between two
+    samples) and sech envelopes of widths N/16 to N, each at 16 sizes in [1/2, 1)."""
+    mu = np.fft.ifftshift(np.arange(N) - N // 2)
+    out = [np.ones(N), 1j * np.ones(N), (1 + 1j) * np.ones(N), np.exp(2j * np.pi * 0.3 * mu)]
+    out += [1 / np.cosh(mu / (N / w)) for w in (16, 8, 4, 2, 1)]
+    size = 2.0 ** (np.arange(-16, 0) / 16)
+    return (size[:, None, None] * np.array(out)).reshape(-1, N)
+
+
+def rel(x, y):
+    return np.linalg.norm(x - y, axis=-1) / np.linalg.norm(y, axis=-1)
+
+
+def rhs_extended(D, g0=G0):
+    a = np.fft.ifft(D.astype(L)) * D.shape[-1]
+    return 1j * L(g0) * np.fft.fft((a.real ** 2 + a.imag ** 2) * a) / D.shape[-1]
+
+
+@pytest.mark.parametrize("logN,R", shapes())
+def test_kerr_term_of_short_pulses(builds, tmp_path, logN, R):
+    D = pulses(1 << logN)
+    err = rel(run(builds[logN, R], "rhs", D, tmp_path), rhs_extended(D))
+    assert err.max() <= ULP * 4 * (logN + 2), (int(err.argmax()), float(err.max()))
+
+
+def propagator(D, t):
+    return np.exp((L(-KAPPA / 2) - 1j * L(SIGMA)) * L(t))
+
+
+def rk4ip_extended(D, h, pump):
+    D, h, E = D.astype(L), np.longdouble(h), propagator(D, np.longdouble(h) / 2)
+
+    def F(x):
+        y = rhs_extended(x)
+        y[..., 0] += L(pump)
+        return y
+
+    k1 = E * F(D)
+    k2 = F(E * D + h / 2 * k1)
+    k3 = F(E * D + h / 2 * k2)
+    k4 = F(E * (E * D + h * k3))
+    return E * (E * D + h / 6 * (k1 + 2 * k2 + 2 * k3)) + h / 6 * k4
+
+
+def strang_extended(D, h, pump):
+    D, E = D.astype(L), propagator(D, np.longdouble(h) / 2)
+    into = (E - 1) / (L(-KAPPA / 2) - 1j * L(SIGMA)) * L(pump)
+    D = E * D
+    D[..., 0] += into
+    a = np.fft.ifft(D) * D.shape[-1]
+    D = E * np.fft.fft(a * np.exp(1j * L(G0) * L(h) * (a.real ** 2 + a.imag ** 2))) / D.shape[-1]
+    D[..., 0] += into
+    return D
+
+
+@pytest.mark.parametrize("logN,R", shapes())
+@pytest.mark.parametrize("what,step,phase", [("rk4ip", rk4ip_extended, 0.2),
+                                             ("strang", strang_extended, 0.2)])
+def test_steps_of_short_pulses(builds, tmp_path, logN, R, what, step, phase):
+    """phase: the Kerr phase of the largest sample of each shape's sixteen sizes."""
+    N = 1 << logN
+    for D in np.moveaxis(pulses(N).reshape(16, -1, N), 1, 0):
+        h = phase / (G0 * np.abs(np.fft.ifft(D) * N).max() ** 2)
+        err = rel(run(builds[logN, R], what, D, tmp_path, pump=0.5, h=h), step(D, h, 0.5))
+        assert err.max() <= ULP * 8 * (logN + 4), (int(err.argmax()), float(err.max()))

@@ -537,6 +537,7 @@ struct FixTransform {
         int qc;       // -g |a|^2 is (|a|^2 G) 2^-qc before its shift
         int q;        // scale and bounds of conj(i g |a|^2 a)
         FixBound b;
+        bool over;    // the largest |a|^2, at least 2^(key - 3) units of 2^80, leaves the FP64 range
     };
     CME_DEV static Kerr kerr_scale(const fx (&X)[R], int q, double g, int2* red, int t)
     {
@@ -579,6 +580,7 @@ struct FixTransform {
         k.qc = 2 * qa - 66 + k.ps - eg;
         k.q = qa + k.qc + k.us - 64;
         k.b = {full.bm - less, full.bl - less};
+        k.over = 2 * (SAMPLE - k.up - q) - 3 >= 1024;
         return k;
     }
     // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc
@@ -607,9 +609,10 @@ struct FixTransform {
     // phases take sincos in FP64 (no reduction in that branch: groups of a block may differ).
     // 4 x N = 256 at 4 values per thread: 9.1 -> 4.8 us per split step, most of it the FP64
     // instructions of sincos (about 3500 cycles per value, against about 350).
-    // LG: log2 of the instance's N (this transform's, or that of its cluster).
+    // LG: log2 of the instance's N (this transform's, or that of its cluster).  bad: this thread holds
+    // a sample whose phase is not finite.
     template <int LG>
-    CME_DEV static Kerr kerr_flow(fx (&X)[R], int q, double gh, int2* red, int t)
+    CME_DEV static Kerr kerr_flow(fx (&X)[R], int q, double gh, bool& bad, int2* red, int t)
     {
         constexpr double invN = 1.0 / (1 << LG);
         Kerr k = kerr_scale(X, q, gh * invN, red, t);
@@ -646,8 +649,12 @@ struct FixTransform {
             store(X, -q, a);
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                double sn, cs;
-                sincos(0.5 * gh * (a[j].re * a[j].re + a[j].im * a[j].im), &sn, &cs);
+                const double y = 0.5 * gh * (a[j].re * a[j].re + a[j].im * a[j].im);
+                double sn = 0.0, cs = 0.0;
+                if (isfinite(y))
+                    sincos(y, &sn, &cs);
+                else
+                    bad = true;
                 // conj(expm1(i phi)) / 4 as limbs; the product with a, 2^-5 of it
                 const fl2 w = {fsplit(fix(-sn * sn, 1085 - 61)), fsplit(fix(-sn * cs, 1085 - 61))};
                 const fx c = {fshl(X[j].re, k.up), -fshl(X[j].im, k.up)};

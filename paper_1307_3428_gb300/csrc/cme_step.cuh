@@ -461,6 +461,7 @@ struct Group {
                         sstore(aout + j * P, x[j]);
                 }
                 const typename FT::Kerr k = FT::kerr(X, q, gN, red, tl());
+                bad |= k.over;
                 q = k.q;
                 b = k.b;
             }
@@ -902,6 +903,7 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, C>& grp, FieldState<double, L
                     }
                 }
                 const typename FT::Kerr k = FT::kerr(X, q, gh, grp.red, grp.tl());
+                bad |= k.over;
                 q = k.q - (st == 2);
                 b = k.b;
             }
@@ -1072,7 +1074,9 @@ CME_DEV void fix_strang_kerr(Group<double, LOGN, R, C>& grp, FieldState<double, 
                         sstore(so + j * P, x[j]);
                 }
             }
-            const typename FT::Kerr k = FT::template kerr_flow<LOGN>(X, q, 2.0 * c.g0h, grp.red, grp.tl());
+            const typename FT::Kerr k =
+                FT::template kerr_flow<LOGN>(X, q, 2.0 * c.g0h, bad, grp.red, grp.tl());
+            bad |= k.over;
             q = k.q;
             b = k.b;
         }

@@ -130,3 +130,19 @@ def test_steps_of_short_pulses(builds, tmp_path, logN, R, what, step, phase):
         h = phase / (G0 * np.abs(np.fft.ifft(D) * N).max() ** 2)
         err = rel(run(builds[logN, R], what, D, tmp_path, pump=0.5, h=h), step(D, h, 0.5))
         assert err.max() <= ULP * 8 * (logN + 4), (int(err.argmax()), float(err.max()))
+
+
+@pytest.mark.parametrize("logN,R", shapes())
+@pytest.mark.parametrize("what", ["rk4ip", "strang"])
+def test_overflowing_fields_become_nan(builds, tmp_path, logN, R, what):
+    """A field whose |a|^2 leaves the FP64 range has no result: every mode is NaN or infinite after
+    the step, and instances in the same block keep the bits they have alone."""
+    N = 1 << logN
+    rng = np.random.default_rng(5)
+    D = np.tile(rng.standard_normal((N, 2)).view(complex)[:, 0], (4, 1))
+    D[1] *= 1e200
+    D[3, 1] = 1e155
+    got = run(builds[logN, R], what, D, tmp_path, pump=0.5)
+    assert not np.isfinite(got[[1, 3]]).any()
+    alone = run(builds[logN, R], what, D[:1], tmp_path, pump=0.5)
+    np.testing.assert_array_equal(got[[0, 2]], np.concatenate([alone, alone]))

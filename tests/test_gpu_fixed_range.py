@@ -1,0 +1,30 @@
+"""The ends of the FP64 range in the fixed-point kernels: what is not finite is reported, by both
+integrators, with and without clusters, and zeros stay zeros."""
+import numpy as np
+import pytest
+
+from paper_1307_3428_gb300 import cme
+
+pytestmark = pytest.mark.gpu
+PLANS = [(16, {}), (64, {"radix": 8}), (512, {}), (1024, {}), (4096, {"cluster": 1}),
+         (2048, {"cluster": 4}), (4096, {"cluster": 8})]
+
+
+def batch(N, D, A_in=0.7, **kw):
+    return cme.Batch([cme.Instance(N, np.ones(N), np.zeros(N), 1.3, 0.5, A_in, 1.0, d) for d in D],
+                     **kw)
+
+
+@pytest.mark.parametrize("N,kw", PLANS)
+@pytest.mark.parametrize("integ", [cme.RK4IP, cme.STRANG])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 1e155, 1e200])
+def test_non_finite_steps_are_reported(N, kw, integ, bad):
+    rng = np.random.default_rng(N)
+    D = rng.standard_normal((3, N, 2)).view(complex)[..., 0] / np.sqrt(N)
+    b = batch(N, D, integrator=integ, **kw)
+    D[1, 1] = bad
+    b.set_state(D.reshape(-1))
+    b.step(1e-3, 1)
+    assert list(b.status()) == [0, 1, 0]
+    got = b.get_state().reshape(3, N)
+    assert not np.isfinite(got[1]).any() and np.isfinite(got[[0, 2]]).all()

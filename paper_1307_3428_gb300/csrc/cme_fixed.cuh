@@ -477,12 +477,19 @@ struct FixTransform {
             X[j] = {fix(x[j].re, c0), fix(x[j].im, c0)};
         return {bad ? POISON : LIM - B0 - E + 1023 + pre, {bm + LIM - B0, bl + LIM - B0}};
     }
-    // v 2^(1085 - c0), rounded; |result| < 2^62
+    // v 2^(1085 - c0), rounded; |result| < 2^62.  SUB: c0 may be below 64, where zero and subnormal
+    // numbers have to be told from normal ones of the smallest exponent; above, both round to 0.
+    template <bool SUB = false>
     CME_DEV static long long fix(double v, int c0)
     {
         const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-        const int sh = min(c0 - 1 - (int)((hi >> 20) & 0x7ffu), 63);   // one more bit, rounded off
-        const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+        int e = (int)((hi >> 20) & 0x7ffu);
+        unsigned mh = (hi & 0xfffffu) | 0x100000u;
+        if (SUB && e == 0) {
+            e = 1;
+            mh &= 0xfffffu;
+        }
+        const int sh = min(c0 - 1 - e, 63);   // one more bit, rounded off
         const unsigned long long m =
             ((unsigned long long)__funnelshift_l(lo, mh, 10) << 32) | (lo << 10);
         const long long a = (long long)(((m >> sh) + 1) >> 1);
@@ -580,7 +587,7 @@ struct FixTransform {
         k.qc = 2 * qa - 66 + k.ps - eg;
         k.q = qa + k.qc + k.us - 64;
         k.b = {full.bm - less, full.bl - less};
-        k.over = 2 * (SAMPLE - k.up - q) - 3 >= 1024;
+        k.over = 2 * (SAMPLE - qa) - 3 >= 1024;
         return k;
     }
     // X becomes conj(i g |a|^2 a) 2^k.q; returns -g |a|^2 2^k.qc

@@ -926,7 +926,8 @@ CME_DEV void fix_rk4ip_step(Group<double, LOGN, R, C>& grp, FieldState<double, L
         }
         if (grp.t == 0) {
             const int c0 = 1085 - q - (st == 2);
-            X[0] = fadd(X[0], {FT::fix(pump.re, c0), FT::fix(pump.im, c0)});
+            X[0] = fadd(X[0], {FT::template fix<true>(pump.re, c0),
+                               FT::template fix<true>(pump.im, c0)});
         }
         if constexpr (STAGES) {
             if (so && st < 3) {

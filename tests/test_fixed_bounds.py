@@ -146,3 +146,24 @@ def test_overflowing_fields_become_nan(builds, tmp_path, logN, R, what):
     assert not np.isfinite(got[[1, 3]]).any()
     alone = run(builds[logN, R], what, D[:1], tmp_path, pump=0.5)
     np.testing.assert_array_equal(got[[0, 2]], np.concatenate([alone, alone]))
+
+
+@pytest.mark.parametrize("logN,R", shapes())
+def test_unpumped_zero_field_stays_zero(builds, tmp_path, logN, R):
+    D = np.zeros((3, 1 << logN), complex)
+    assert not run(builds[logN, R], "rk4ip", D, tmp_path, steps=3).any()
+    D[1, 1] = 1e-160           # its Kerr term lies far below the range: no mixing into mode 0
+    got = run(builds[logN, R], "rk4ip", D, tmp_path, steps=3)
+    assert got[1, 1] != 0 and not np.delete(got[1], 1).any() and not got[[0, 2]].any()
+
+
+@pytest.mark.parametrize("pump", [1e-300, 3e-308, 1e-310])
+def test_smallest_pumps(builds, tmp_path, pump):
+    """A pump near the end of the range (its half step subnormal) on a zero field: h pump after a
+    short step, to the spacing of the range's end."""
+    h = 1e-3
+    for logN, R in ((4, 2), (6, 8), (9, 4)):
+        got = run(builds[logN, R], "rk4ip", np.zeros((1, 1 << logN), complex), tmp_path, pump=pump,
+                  h=h)[0]
+        assert abs(got[0] - pump * h) <= 2e-3 * pump * h + 8 * 2.0 ** -1074
+        assert not got[1:].any()

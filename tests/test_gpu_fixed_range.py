@@ -28,3 +28,15 @@ def test_non_finite_steps_are_reported(N, kw, integ, bad):
     assert list(b.status()) == [0, 1, 0]
     got = b.get_state().reshape(3, N)
     assert not np.isfinite(got[1]).any() and np.isfinite(got[[0, 2]]).all()
+
+
+@pytest.mark.parametrize("N,kw", PLANS)
+@pytest.mark.parametrize("integ", [cme.RK4IP, cme.STRANG])
+def test_unpumped_zero_fields_stay_zero(N, kw, integ):
+    D = np.zeros((3, N), complex)
+    D[1, 1] = 1e-160
+    b = batch(N, D, A_in=0.0, integrator=integ, **kw)
+    b.step(1e-3, 3)
+    got = b.get_state().reshape(3, N)
+    assert list(b.status()) == [0, 0, 0]
+    assert got[1, 1] != 0 and not np.delete(got[1], 1).any() and not got[[0, 2]].any()

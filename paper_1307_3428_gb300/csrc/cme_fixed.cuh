@@ -662,14 +662,15 @@ struct FixTransform {
                     sincos(y, &sn, &cs);
                 else
                     bad = true;
-                // conj(expm1(i phi)) / 4 as limbs; the product with a, 2^-5 of it
-                const fl2 w = {fsplit(fix(-sn * sn, 1085 - 61)), fsplit(fix(-sn * cs, 1085 - 61))};
-                const fx c = {fshl(X[j].re, k.up), -fshl(X[j].im, k.up)};
-                const fx b = fcmul4(c, w);
-                X[j] = {fshift(b.re, 1), fshift(b.im, 1)};
+                // a times conj(expm1(i phi)) / 2, whose modulus is at most 1
+                const fl2 w = {fsplit(fix(-sn * sn, 1085 - 62)), fsplit(fix(-sn * cs, 1085 - 62))};
+                X[j] = fcmul1({fshl(X[j].re, k.up), -fshl(X[j].im, k.up)}, w);
             }
-            k.q = q + k.up - 5 + LG;
-            k.b = {61 - 4, 61 - 4 + LOGN};
+            // |a expm1(i phi)| / 2 <= |a| min(1, phi / 2): L1 is at most N |a|max, and at most
+            // 2^(f - 1) |a|max sum (|a| / |a|max)^3 with phi < 2^f, the sum from the scale's bounds
+            const int f = -2 - sh;
+            k.q = q + k.up - 1 + LG;
+            k.b = {SAMPLE, SAMPLE + min(LOGN, f - 1 + k.b.bl - k.b.bm)};
             const int less = max(headroom<false>(k.b) - LIM, 0);
 #pragma unroll
             for (int j = 0; j < R; ++j)

@@ -122,9 +122,11 @@ def strang_extended(D, h, pump):
 
 @pytest.mark.parametrize("logN,R", shapes())
 @pytest.mark.parametrize("what,step,phase", [("rk4ip", rk4ip_extended, 0.2),
-                                             ("strang", strang_extended, 0.2)])
+                                             ("strang", strang_extended, 0.2),
+                                             ("strang", strang_extended, 5.0)])
 def test_steps_of_short_pulses(builds, tmp_path, logN, R, what, step, phase):
-    """phase: the Kerr phase of the largest sample of each shape's sixteen sizes."""
+    """phase: the Kerr phase of the largest sample of each shape's sixteen sizes (the split step's
+    series ends at 1)."""
     N = 1 << logN
     for D in np.moveaxis(pulses(N).reshape(16, -1, N), 1, 0):
         h = phase / (G0 * np.abs(np.fft.ifft(D) * N).max() ** 2)

@@ -43,10 +43,12 @@ def test_rhs_of_short_pulses(N, R):
 @pytest.mark.parametrize("N,kw", [(32, {}), (64, {"radix": 8}), (512, {"radix": 8}), (1024, {}),
                                   (4096, {"cluster": 1}), (256, {"radix": 8, "cluster": 2}),
                                   (2048, {"cluster": 4}), (4096, {"cluster": 8})])
-@pytest.mark.parametrize("integ,step", [(cme.RK4IP, rk4ip_extended), (cme.STRANG, strang_extended)])
-def test_steps_of_short_pulses(N, kw, integ, step):
+@pytest.mark.parametrize("integ,step,phase", [(cme.RK4IP, rk4ip_extended, 0.2),
+                                              (cme.STRANG, strang_extended, 0.2),
+                                              (cme.STRANG, strang_extended, 5.0)])
+def test_steps_of_short_pulses(N, kw, integ, step, phase):
     for D in np.moveaxis(pulses(N).reshape(16, -1, N), 1, 0):
-        h = float(0.2 / (G0 * np.abs(np.fft.ifft(D) * N).max() ** 2))
+        h = float(phase / (G0 * np.abs(np.fft.ifft(D) * N).max() ** 2))
         b = batch(D, integrator=integ, **kw)
         b.step(h, 1)
         err = rel(modes(b.get_state(), N), step(D, h, PUMP))

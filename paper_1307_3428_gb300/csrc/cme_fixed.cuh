@@ -323,7 +323,7 @@ struct GroupReduce {
 
 // Fixed-point transform of one group; the passes, exchanges and twiddles are those of
 // Transform, inverse direction only (the forward transform is conj(inverse(conj(.)))).
-template <int LOGN, int R, bool WARP>
+template <int LOGN, int R, bool WARP, bool CLUSTER = false>
 struct FixTransform {
     using PL = Plan<LOGN, R>;
     using TF = Transform<double, LOGN, R, WARP>;   // exchange layout
@@ -340,26 +340,57 @@ struct FixTransform {
     static constexpr int KB = LIM - ilog2(PL::radix(0)) < 59 ? LIM - ilog2(PL::radix(0)) : 59;
     using GRd = GroupReduce<P>;
 
-    static constexpr int OUT = HB * (NS - 1);   // the result of a run is X 2^OUT
+    static constexpr int OUT = HB * (NS - 1);   // the result of a run is X 2^(OUT - lift)
 
     // Bits that an input of bounds b reaches, over the passes: at most LIM before a run.  KERR: the
     // result goes to the Kerr term, so that it counts LIM - SAMPLE bits more than the passes.  (Where
     // the last pass is the largest, on short pulses with their flat spectra, it left samples of up
     // to 2^62, and the Kerr term overflowed: error of order 1.  Other fields keep their scale.)
-    template <bool KERR>
+    // FROM: the first pass that counts.
+    template <bool KERR, int FROM = 0>
     CME_DEV static int headroom(FixBound b)
     {
-        int g = b.bm + ilog2(PL::radix(0)), h = min(b.bl, g);
+        int g = b.bm + ilog2(PL::radix(0)), h = FROM == 0 ? min(b.bl, g) : -(1 << 20);
 #pragma unroll
         for (int s = 1; s < NS; ++s) {
             g += ilog2(PL::radix(s));
-            h = max(h, min(b.bl, g) - s * HB);
+            if (s >= FROM)
+                h = max(h, min(b.bl, g) - s * HB);
         }
         if constexpr (KERR && LIM > SAMPLE)
             h = max(h, min(b.bl, g) - OUT + (LIM - SAMPLE));
         return h;
     }
-    // bits of the result's modulus
+    // Where the bounds grow less than the passes scale down, the samples lie bits below the limit, and
+    // the rounding of the last passes lies above FP64's.  Transforms of many passes, and those of a
+    // cluster's blocks, therefore shift their values left before the passes s of lifts(s), by what
+    // the passes from s - 1 on leave free (`up`; lift returns their sum).  Error of the modes below
+    // 1e-4 after an RK4IP step of a comb (tests/test_fixed_bounds.py), relative to that of FP64
+    // instructions, without and with it: N = 128 at 2 values per thread 1.4 and 0.4, N = 1024 1.7 and
+    // 0.9, N = 2048 1.3 and 1.0, N = 4096 2.2 and 1.55, clusters of 2 ... 8 blocks 1.0 to 2.6 and 0.8 to
+    // 1.0 at N = 2048, 2.0 to 3.7 and 1.35 to 1.45 at N = 4096; all modes together 1.00.  What is left
+    // at N = 4096 is the unit of the Kerr term, set by the envelope's peak, on the samples beside it.
+    // us per RK4IP step without and with: N = 128 x 300 8.6 / 8.7, N = 1024 x 300 36.2 / 36.9,
+    // N = 2048 x 150 45.9 / 46.2, N = 4096 x 150 107.6 / 104.1, x 64 (clusters) 72.6 / 73.1.
+    CME_HD static constexpr bool lifts(int s)
+    {
+        return R == 2 ? LOGN == 7 && (s == 3 || s == 5) : (LOGN >= 10 || CLUSTER) && s >= 2;
+    }
+    template <bool KERR, int s = 1>
+    CME_DEV static int lift(FixBound b, int (&up)[NS], int sum = 0)
+    {
+        if constexpr (s < NS) {
+            up[s] = 0;
+            if constexpr (lifts(s)) {
+                up[s] = min(max(LIM - headroom<KERR, s - 1>(b) - sum, 0), 15);
+                sum += up[s];
+            }
+            return lift<KERR, s + 1>(b, up, sum);
+        } else {
+            return sum;
+        }
+    }
+    // bits of the modulus of a run's result, before its shift
     CME_DEV static int out_bits(FixBound b) { return min(b.bl, b.bm + LOGN) - OUT; }
 
     template <int s, class TW>
@@ -407,8 +438,13 @@ struct FixTransform {
     }
     template <int s, class TW>
     CME_DEV static void run_from(fx (&x)[R], const TW& tw, const Xbuf<double>& buf, int& par,
-                                 const typename TF::Addr& ad)
+                                 const typename TF::Addr& ad, const int (&up)[NS])
     {
+        if constexpr (lifts(s)) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                x[j] = {fshl(x[j].re, up[s]), fshl(x[j].im, up[s])};
+        }
         pass<s>(x, tw);
         if constexpr (s + 1 < NS) {
             cx<double> y[R];
@@ -420,14 +456,14 @@ struct FixTransform {
             for (int j = 0; j < R; ++j)
                 x[j] = {__double_as_longlong(y[j].re), __double_as_longlong(y[j].im)};
             par ^= 1;
-            run_from<s + 1>(x, tw, buf, par, ad);
+            run_from<s + 1>(x, tw, buf, par, ad, up);
         }
     }
     template <class TW>
     CME_DEV static void run(fx (&x)[R], const TW& tw, const Xbuf<double>& buf, int& par,
-                            const typename TF::Addr& ad)
+                            const typename TF::Addr& ad, const int (&up)[NS])
     {
-        run_from<0>(x, tw, buf, par, ad);
+        run_from<0>(x, tw, buf, par, ad, up);
     }
 
     // Scale of a group's FP64 values: X = x 2^q, bounds of X.  q = POISON: a value is not finite.

@@ -110,7 +110,7 @@ struct Group {
     static constexpr bool TW_SMEM = !TW_REGS && twiddles_in_smem(sizeof(T), LOGN - LC);
     // FP64 transforms run in fixed point (cme_fixed.cuh)
     static constexpr bool FIX = sizeof(T) == 8;
-    using FT = FixTransform<LOGN - LC, R, (Plan<LOGN - LC, R>::P <= 32)>;
+    using FT = FixTransform<LOGN - LC, R, (Plan<LOGN - LC, R>::P <= 32), (C > 1)>;
     using TW = std::conditional_t<
         FIX, FixTwiddles<LOGN - LC, R, TW_REGS, C>,
         std::conditional_t<TW_SMEM, TwiddlesSmem<T, LOGN - LC, R, C>,
@@ -249,9 +249,11 @@ struct Group {
     CME_DEV int fix_inverse(fx (&X)[R], int& q, FixBound b, bool& bad, int d)
     {
         if constexpr (C == 1) {
-            FT::run(X, tw, buf, par, ad);
-            q -= FT::OUT;
-            return FT::out_bits(b);
+            int ups[FT::NS];
+            const int up = FT::template lift<TO_KERR>(b, ups);
+            FT::run(X, tw, buf, par, ad, ups);
+            q += up - FT::OUT;
+            return FT::out_bits(b) + up;
         } else {
             constexpr int G = CF::G, PC = CF::PC;
             int bits = 0;
@@ -284,17 +286,18 @@ struct Group {
                     cnt += (1u << 20) >> min(top - (ls[c] - (qs[c] - q)), 31);
                 b = {bm, top + 32 - __clz((int)(cnt - 1)) - 20};
                 const int s = FT::LIM - FT::template headroom<false>(b);
-                const int use = s < 0 || s > 3 ? s : 0;
-                q += use;
-                b.bm += use;
-                b.bl += use;
+                q += s;
+                b.bm += s;
+                b.bl += s;
 #pragma unroll
                 for (int j = 0; j < R; ++j)
                     X[j] = align_to(X[j], qs[j % C] - q);
             }
-            FT::run(X, tw, buf, par, ad);
-            q -= FT::OUT;
-            bits = FT::out_bits(b);
+            int ups[FT::NS];
+            const int up = FT::template lift<TO_KERR>(b, ups);
+            FT::run(X, tw, buf, par, ad, ups);
+            q += up - FT::OUT;
+            bits = FT::out_bits(b) + up;
             if (d == 0) {
                 if (rank != 0) {   // block 0's twiddles are 1
 #pragma unroll

@@ -169,3 +169,60 @@ def test_smallest_pumps(builds, tmp_path, pump):
                   h=h)[0]
         assert abs(got[0] - pump * h) <= 2e-3 * pump * h + 8 * 2.0 ** -1074
         assert not got[1:].any()
+
+
+def combs(N, rng, n):
+    """Sech envelopes of a random time and width on a continuous wave and noise."""
+    mu = np.fft.ifftshift(np.arange(N) - N // 2)
+    W = rng.uniform(N / 24, N / 8, (n, 1))
+    D = rng.standard_normal((n, N, 2)).view(complex)[..., 0] * 10.0 ** rng.uniform(-8, -6, (n, 1))
+    D += (rng.uniform(0.5, 1.5, (n, 1)) / W / np.cosh(np.minimum(np.abs(mu / W), 300)) *
+          np.exp(2j * np.pi * rng.uniform(0, 1, (n, 1)) * mu))
+    D[:, 0] += rng.uniform(0.3, 1.5, n) * np.exp(2j * np.pi * rng.uniform(0, 1, n))
+    return D
+
+
+def small_mode_errors(D, got, h, pump):
+    """Root mean square error over the modes below 1e-4, of `got` and of FP64 arithmetic."""
+    want = rk4ip_extended(D, h, pump)
+    E, e1, e2 = (propagator(D, np.longdouble(h) / 2), propagator(D, np.longdouble(h) / 2) - 1,
+                 propagator(D, h) - 1)
+    E, e1, e2, N = complex(E), complex(e1), complex(e2), D.shape[-1]
+
+    def F(x):
+        a = np.fft.ifft(x) * N
+        y = 1j * G0 * (np.fft.fft((a.real ** 2 + a.imag ** 2) * a) / N)
+        y[..., 0] += pump
+        return y
+
+    k1 = E * F(D)
+    k2 = F(D + (e1 * D + h / 2 * k1))
+    k3 = F(D + (e1 * D + h / 2 * k2))
+    k4 = F(D + (e2 * D + h * E * k3))
+    plain = D + (e2 * D + h / 6 * (E * (k1 + 2 * k2 + 2 * k3) + k4))
+    small = np.abs(D) < 1e-4
+    return [float(np.sqrt(np.mean(np.abs((x - want)[small]) ** 2))) for x in (got, plain)]
+
+
+@pytest.mark.parametrize("logN,R", [s for s in shapes() if s[0] >= 4])
+def test_small_modes_of_an_rk4ip_step(builds, tmp_path, logN, R):
+    """One scale per instance leaves modes far below the pumped one fewer bits than FP64 numbers
+    have.  What counts is the error of a step on them: at most twice that of FP64 arithmetic with
+    numpy's transforms."""
+    N = 1 << logN
+    D = combs(N, np.random.default_rng(logN), 128 if N < 1024 else 32)
+    h = 1e-3 if N <= 128 else 5e-4 if N <= 512 else 2e-4
+    fixed, plain = small_mode_errors(D, run(builds[logN, R], "rk4ip", D, tmp_path, pump=1.5, h=h),
+                                     h, 1.5)
+    assert fixed <= 2 * plain
+
+
+@pytest.mark.parametrize("logN,R", [(9, 4), (9, 8), (12, 8)])
+def test_increment_unit(builds, tmp_path, logN, R):
+    """A continuous wave of 1.3 with modes of 1e-6, h = 2e-4: the increment, about 1e-3, is held to
+    2^-60 of itself, so the small modes end within 2e-21 (FP64 instructions: 1.6e-21 to 4.9e-21)."""
+    rng = np.random.default_rng(1)
+    D = 1e-6 * rng.standard_normal((16, 1 << logN, 2)).view(complex)[..., 0]
+    D[:, 0] += 1.2 + 0.4j
+    got = run(builds[logN, R], "rk4ip", D, tmp_path, pump=0.5, h=2e-4)
+    assert small_mode_errors(D, got, 2e-4, 0.5)[0] <= 2e-21

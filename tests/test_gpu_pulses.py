@@ -40,7 +40,8 @@ def test_rhs_of_short_pulses(N, R):
     assert err.max() <= ULP * 4 * (np.log2(N) + 2), int(err.argmax())
 
 
-@pytest.mark.parametrize("N,kw", [(32, {}), (64, {"radix": 8}), (512, {"radix": 8}), (1024, {}),
+@pytest.mark.parametrize("N,kw", [(16, {}), (32, {}), (64, {"radix": 8}), (128, {}),
+                                  (512, {"radix": 8}), (1024, {}), (1024, {"radix": 4}),
                                   (4096, {"cluster": 1}), (256, {"radix": 8, "cluster": 2}),
                                   (2048, {"cluster": 4}), (4096, {"cluster": 8})])
 @pytest.mark.parametrize("integ,step,phase", [(cme.RK4IP, rk4ip_extended, 0.2),

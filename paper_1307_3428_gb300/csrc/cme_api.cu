@@ -119,8 +119,14 @@ bool shape_compiled(int logN, int R)
     return false;
 }
 
-// The shapes a caller may name: 2 values per thread at N = 16 and 32 are the library's choice only.
-bool radix_on_request(int logN, int R) { return shape_compiled(logN, R) && (R != 2 || logN >= 6); }
+// The shapes a caller may name.  2 values per thread at N = 16 and 32 are refused as a radix by
+// itself, and accepted where a plan that cme_batch_plan returned is named with its instances per
+// block (the library chooses that shape for FP64 groups only).
+bool radix_on_request(int logN, int R, int prec, int inst_per_cta)
+{
+    return shape_compiled(logN, R) &&
+           (R != 2 || logN >= 6 || (prec == PREC_FP64 && inst_per_cta > 0));
+}
 
 // Values per thread: 8 (N = 4: 4), except FP32 N >= 2048, which take 16: with their twiddles
 // in shared memory and their propagators in registers that measured 11.7 against 13.3 us per
@@ -355,7 +361,8 @@ int plan_batch(cme_batch b, const cme_options& o)
             R = 8;
         if (R > g.N)
             R = g.N;
-        if (!(o.radix ? radix_on_request(g.logN, R) : shape_compiled(g.logN, R)))
+        if (!(o.radix ? radix_on_request(g.logN, R, b->prec, o.inst_per_cta)
+                      : shape_compiled(g.logN, R)))
             return fail(CME_ERR_INVALID_ARG, "launch plan: radix %d not available for N=%d", R, g.N);
         g.R = R;
         g.G = inst_per_block(g.N, R, o.inst_per_cta, g.count);
@@ -683,7 +690,7 @@ int cme_batch_create(const cme_instance* v, int count, const cme_options* opt, v
             continue;
         }
         const int R = std::min(o.radix ? o.radix : default_radix(g.logN, b->prec), N);
-        if (!radix_on_request(g.logN, R) || o.persistent < 0 || o.persistent > 2 ||
+        if (!radix_on_request(g.logN, R, b->prec, o.inst_per_cta) || o.persistent < 0 || o.persistent > 2 ||
             !(o.cluster == 0 || o.cluster == 1 || o.cluster == 2 || o.cluster == 4 ||
               o.cluster == 8)) {
             cme_batch_destroy(b);
@@ -1396,7 +1403,7 @@ int cme_autotune(cme_batch b, double h, long probe_steps, cme_options* plan_out)
         for (int R : {2, 4, 8, 16}) {
             if (R > g.N || !shape_compiled(g.logN, R))
                 continue;
-            if (!radix_on_request(g.logN, R)) {   // reachable as the library's choice, or not at all
+            if (!radix_on_request(g.logN, R, b->prec, 0)) {   // reachable as the library's choice, or not at all
                 cme_options o = base;
                 o.radix = 0;
                 o.inst_per_cta = 0;

@@ -6,10 +6,14 @@ namespace cme {
 #define CME_LARGE_ROWS(X) X(7, 8) X(8, 8) X(9, 8) X(8, 4) X(9, 4)
 #define CME_LARGE_COLS(X) X(8, 8) X(9, 8) X(8, 4) X(9, 4)
 
-// Packed arithmetic for 2^15 <= N <= 2^18, scalar (kern_large_fp32_scalar.cu) for the others.
-// us per step, scalar / packed: 2^13 17.2 / 17.8, 8 instances 20.5 / 23.7; 2^14 18.5 / 18.7;
-// 2^15 20.5 / 20.2; 2^16 28.5 / 28.1; 2^17 29.8 / 29.4; 2^18 x 3 114.6 / 114.2; 2^19 98.6 / 102.4;
-// 2^20 152.1 / 154.0 (columns of N1 = 1024: 178 registers, two blocks per SM where 164 leave three).
+// Packed arithmetic for 2^15 <= N <= 2^18, scalar (kern_large_fp32_scalar.cu) for the others: a rule on
+// N alone, so that the grid-barrier kernel below, which is packed, repeats the sequence's bits.
+// us per step, scalar / packed: 2^13 17.1 / 16.8, 8 instances 21.1 / 24.5, 9 21.4 / 28.8; 2^14 18.4 / 17.9,
+// 4 instances 23.3 / 23.3, 12 39.4 / 39.7; 2^15 20.4 / 19.3, 2 instances 26.1 / 27.3, 3 25.3 / 24.7,
+// 4 27.0 / 25.3, 6 44.6 / 47.0, 8 41 / 38.7; 2^16 29.9 / 30.5, 2 instances 28.9 / 27.8, 3 54.9 / 50.5;
+// 2^17 29.9 / 29.2, 2 instances 62.5 / 61.2; 2^18 45.5 / 45.6, 3 instances 114.5 / 114.2; 2^19 96.2 /
+// 101.8; 2^20 151.8 / 153.1 (columns of N1 = 1024: 178 registers, two blocks per SM where 164 leave
+// three).
 static bool packed(const LargeArgs& a)
 {
     const int logN = a.logN1 + a.logN2;

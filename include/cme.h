@@ -45,8 +45,13 @@ extern "C" {
 #define CME_ERR_STATE (-7)         /* call out of order (e.g. instance without a field) */
 
 /* ---- options ----------------------------------------------------------------------- */
-#define CME_FP64 0 /* FP64 field and propagators; transforms, Kerr term and RK4IP stages to FP64
-                      accuracy, computed in 64-bit fixed point with one scale per instance */
+#define CME_FP64 0 /* FP64 field and propagators; transforms and Kerr term to FP64 accuracy, computed
+                      in 64-bit fixed point with one scale per transform: an instance, or each
+                      block of its cluster (cluster > 1), or each row or column (N > 4096).
+                      RK4IP stages in fixed point too, except with per-mode Kerr coefficients
+                      and for N > 4096, where they are FP64 instructions.  Whole fields are as
+                      accurate as with FP64 instructions; modes below 1e-4 of a comb's largest
+                      at N = 4096 are up to 1.5 times less so */
 #define CME_FP32 1 /* FP32 field, transforms and Kerr term; propagators computed in FP64 and
                       applied as small increments; state kept as a compensated FP32 pair */
 
@@ -322,7 +327,7 @@ int cme_eval_rhs(cme_batch b, double* out, int where);
  * instances per block) that cme_batch_create chooses for an FP64 RK4IP batch of these
  * instances under default options before its choice of thread-block clusters: the result is
  * bit for bit that of such a batch created with cluster = 1.  Where the default batch spreads
- * N = 2048 or 4096 instances over clusters, the two agree to rounding only.  All pointers are
+ * N = 4096 instances over clusters, the two agree to rounding only.  All pointers are
  * device memory owned by the caller:
  *   d_kappa, d_omega  N * count doubles each: kappa_mu and omega_mu per instance, centred;
  *   d_inst            5 * count doubles: (g0, kappa_ext, Re A_in, Im A_in, sigma) per instance;

@@ -723,7 +723,16 @@ int cme_batch_create(const cme_instance* v, int count, const cme_options* opt, v
     b->E = A(T * b->elem);
     b->e1 = A(T * b->elem);
     b->e2 = A(T * b->elem);
-    if (b->prec == PREC_FP64 && b->method == METHOD_RK4IP)
+    // the limbs of E: fixed-point RK4IP stages, which four-step groups and groups with per-mode Kerr
+    // coefficients do not run
+    bool stages = false;
+    for (const auto& g : b->groups) {
+        bool kerr = false;
+        for (int i = g.first; i < g.first + g.count; ++i)
+            kerr |= !v[i]->g0mu.empty();
+        stages |= !g.large && !kerr;
+    }
+    if (b->prec == PREC_FP64 && b->method == METHOD_RK4IP && stages)
         b->Ef = A(T * 16);
     b->diag = A(T * b->elem);
     b->kappa = (double*)A(T * 8);

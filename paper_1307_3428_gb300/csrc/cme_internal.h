@@ -21,7 +21,7 @@ struct StepArgs {
     const void* E;          // exp(L h/2) per mode                (RK4IP)
     const void* e1;         // expm1(L h/2) per mode              (RK4IP and Strang)
     const void* e2;         // expm1(L h) per mode                (RK4IP)
-    const void* Ef;         // FP64 RK4IP: limbs of E per mode (cme_fixed.cuh), else null
+    const void* Ef;         // limbs of E per mode (cme_fixed.cuh) for fixed-point RK4IP stages
     const void* tw;         // twiddle table exp(2 pi i k / N), k < N
     const double2* pump;    // per-instance pump sqrt(kappa_ext) A_in (group-relative)
     const double2* cpump;   // per-instance Strang pump increment over h/2
@@ -134,7 +134,7 @@ struct PropArgs {
     void* E;
     void* e1;                 // null: skipped
     void* e2;
-    void* Ef;                 // FP64 RK4IP: limbs of E (int4 per mode), null: skipped
+    void* Ef;                 // limbs of E (int4 per mode), null: skipped
     void* e1h;                // Strang: expm1(L h/2)
     double2* cpump;           // Strang pump increment per instance
     double2* cpump2;          // the same over h (null: not computed)

@@ -40,3 +40,26 @@ def test_unpumped_zero_fields_stay_zero(N, kw, integ):
     got = b.get_state().reshape(3, N)
     assert list(b.status()) == [0, 0, 0]
     assert got[1, 1] != 0 and not np.delete(got[1], 1).any() and not got[[0, 2]].any()
+
+
+def test_per_mode_kerr_batches_hold_no_stage_tables():
+    """The fixed-point stages' propagator (16 bytes per mode) is held only where stages run on it: a
+    batch with per-mode Kerr coefficients needs 8 bytes per mode for those and not more."""
+    torch = pytest.importorskip("torch")
+    N, count = 256, 256
+
+    def held(kerr):
+        insts = [cme.Instance(N, np.ones(N), np.zeros(N), 1.0, 0.5, 0.7, 1.0,
+                              np.zeros(N, complex), None, kerr)] * count
+        before = torch.cuda.memory_allocated()
+        b = cme.Batch(insts)
+        used = torch.cuda.memory_allocated() - before
+        b.close()
+        return used
+
+    cme.use_torch_allocator()
+    try:
+        plain, kerr = held(None), held(np.linspace(0.9, 1.1, N))
+    finally:
+        cme.load().cme_set_allocator(cme.ALLOC_FN(), cme.FREE_FN(), None)
+    assert 0 < kerr <= plain - 8 * N * count + 4096

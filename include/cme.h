@@ -330,6 +330,9 @@ int cme_eval_rhs(cme_batch b, double* out, int where);
  * N = 4096 instances over clusters, the two agree to rounding only.  All pointers are
  * device memory owned by the caller:
  *   d_kappa, d_omega  N * count doubles each: kappa_mu and omega_mu per instance, centred;
+ *                     kappa_mu >= 0 as in cme_create, which this call cannot check; a gain of up
+ *                     to 1.2 per half step, exp(-kappa_mu h / 4), integrates too, and a mode with
+ *                     more comes back as NaN;
  *   d_inst            5 * count doubles: (g0, kappa_ext, Re A_in, Im A_in, sigma) per instance;
  *   d_field           2 * N * count doubles (in/out): rotating-frame field, interleaved, centred.
  * Work is enqueued on cuda_stream (NULL: the legacy default stream) and the call returns without

@@ -65,7 +65,11 @@ __global__ void prop_kernel(PropArgs a)
     const double Li = a.omega[m] - a.sigma[i];
     const double hh = 0.5 * a.h;
     const double2 e1 = cexpm1(Lr * hh, Li * hh);
-    const double2 e2 = cexpm1(Lr * a.h, Li * a.h);
+    double2 e2 = cexpm1(Lr * a.h, Li * a.h);
+    // The fixed-point stages take |E| <= 1 (loss); their bounds have room for a gain of 1.2.  A
+    // larger one would overflow without a trace, so that the mode becomes NaN instead.
+    if (a.Ef && Lr * hh > 0.1823)   // log 1.2
+        e2.x = e2.y = __longlong_as_double(0x7ff8000000000000LL);
     put<V>(a.E, m, make_double2(e1.x + 1.0, e1.y));
     if (a.e1)
         put<V>(a.e1, m, e1);

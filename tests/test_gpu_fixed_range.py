@@ -63,3 +63,43 @@ def test_per_mode_kerr_batches_hold_no_stage_tables():
     finally:
         cme.load().cme_set_allocator(cme.ALLOC_FN(), cme.FREE_FN(), None)
     assert 0 < kerr <= plain - 8 * N * count + 4096
+
+
+@pytest.mark.parametrize("N", [16, 64, 512, 4096])
+def test_gain_through_the_entry_point_without_allocation(N):
+    """cme_rk4ip_noalloc cannot check kappa on the host: a gain of up to 1.2 per half step integrates as
+    in FP64, and a larger one is reported by NaN, not by a finite field."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(N)
+    D = rng.standard_normal((N, 2)).view(complex)[:, 0] / np.sqrt(N)
+    h = 2e-3
+
+    def run(kappa):
+        dev = [torch.tensor(v, dtype=torch.float64, device="cuda")
+               for v in (np.full(N, kappa), np.zeros(N), [1.3, 1.0, 0.5, 0.0, 1.0],
+                         D.view(float).copy())]
+        cme.rk4ip_noalloc(N, 1, h, 2, *(v.data_ptr() for v in dev),
+                          torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        return dev[3].cpu().numpy().view(complex)
+
+    L = np.clongdouble
+    for kappa in (-1.0, -360.0):
+        E = np.exp((L(-kappa / 2) - 1j) * L(h) / 2)
+        x = np.fft.ifftshift(D).astype(L)
+
+        def F(y):
+            a = np.fft.ifft(y) * N
+            z = 1j * L(1.3) * np.fft.fft((a.real ** 2 + a.imag ** 2) * a) / N
+            z[0] += L(0.5)
+            return z
+
+        for _ in range(2):
+            k1 = E * F(x)
+            k2 = F(E * x + h / 2 * k1)
+            k3 = F(E * x + h / 2 * k2)
+            k4 = F(E * (E * x + h * k3))
+            x = E * (E * x + h / 6 * (k1 + 2 * k2 + 2 * k3)) + h / 6 * k4
+        want = np.fft.fftshift(x)
+        assert np.linalg.norm(run(kappa) - want) <= 1e-14 * np.linalg.norm(want)
+    assert np.isnan(run(-2000.0)).all()

@@ -1275,8 +1275,11 @@ CME_DEV void step_body(const StepArgs& a, int first, unsigned char* smem)
 }
 
 // Blocks an SM has to hold (the register limit that sets): FP32 N = 1024 at 8 values per thread
-// three, not the two that 190 registers leave: 400 instances 10.8 -> 6.9 us per step, 900 17.0 ->
-// 13.6 (of that 10 to 13% from the packed arithmetic), a few spilled words against it.
+// three, not the two that 190 registers leave (167, 56 bytes spilled; split step 162, none).  us per
+// step before, with the packed arithmetic in it / now, RK4IP 1 instance 4.04 / 3.60, 300 5.66 / 5.09,
+// 400 10.6 / 6.8, 900 16.9 / 13.5; split step 1.10 / 1.09, 1.87 / 1.65, 2.49 / 2.25, 4.89 / 4.33; with
+// padding modes RK4IP 4.79 / 4.19, 6.15 / 5.64, 12.0 / 7.4, 18.3 / 14.6, split step 1.14 / 1.10,
+// 1.89 / 1.68, 2.42 / 2.31, 4.74 / 4.47.
 template <typename T, int LOGN, int R>
 constexpr int min_blocks() { return sizeof(T) == 4 && LOGN == 10 && R == 8 ? 3 : 1; }
 

@@ -398,8 +398,9 @@ struct FixTransform {
     // bits of the modulus of a run's result, before its shift
     CME_DEV static int out_bits(FixBound b) { return min(b.bl, b.bm + LOGN) - OUT; }
 
+    // up: left shift before this pass (lifts): the bits that it cleared are not lost by the floors.
     template <int s, class TW>
-    CME_DEV static void pass(fx (&x)[R], const TW& tw)
+    CME_DEV static void pass(fx (&x)[R], const TW& tw, int up)
     {
         constexpr int r = PL::radix(s), Q = R / r;
         // Butterflies whose twiddles are all 1 (k = 0; they lead to output 0) floor their products
@@ -409,7 +410,7 @@ struct FixTransform {
         // stay zeros).  Without it: output 0 of N = 4096 off by 4 to 12 times the other outputs'
         // error.
         constexpr bool fix0 = s > 0 && (HB == 2 || r > 2);
-        constexpr int low = HB == 2 ? (3 * r + 4) / 8 : r / 4;
+        const int low = up == 0 ? (HB == 2 ? (3 * r + 4) / 8 : r / 4) : up < HB ? r / 4 : 0;
         bool k0 = false;
         if constexpr (fix0)
             k0 = tw.kst[s] == 0;
@@ -449,8 +450,10 @@ struct FixTransform {
 #pragma unroll
             for (int j = 0; j < R; ++j)
                 x[j] = {fshl(x[j].re, up[s]), fshl(x[j].im, up[s])};
+            pass<s>(x, tw, up[s]);
+        } else {
+            pass<s>(x, tw, 0);
         }
-        pass<s>(x, tw);
         if constexpr (s + 1 < NS) {
             cx<double> y[R];
 #pragma unroll

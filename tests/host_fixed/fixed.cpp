@@ -2,7 +2,7 @@
 // one launch shape (log2 N = CASE_LOGN, CASE_R values per thread) on the host.  Built with overflow checks on every signed
 // operation, it stops at the first sum, product or shift that leaves 64 bits.
 //
-//   fixed rhs|rk4ip|strang <g0> <kappa> <pump> <h> <steps> <fields in> <fields out>
+//   fixed idft|rhs|rk4ip|strang <g0> <kappa> <pump> <h> <steps> <fields in> <fields out>
 //
 // Fields: N complex numbers each, transform order.  Detuning 1, flat dispersion.
 #include <stdio.h>
@@ -35,7 +35,8 @@ static int4 limbs(double re, double im)
 
 int main(int argc, char** argv)
 {
-    const bool rhs = !strcmp(argv[1], "rhs"), strang = !strcmp(argv[1], "strang");
+    const bool idft = !strcmp(argv[1], "idft"), rhs = !strcmp(argv[1], "rhs"),
+               strang = !strcmp(argv[1], "strang");
     const double g0 = atof(argv[2]), kappa = atof(argv[3]), pump = atof(argv[4]), h = atof(argv[5]);
     const int steps = atoi(argv[6]);
     std::vector<int4> tw(N), Ef(N);
@@ -93,7 +94,9 @@ int main(int argc, char** argv)
             fs.load(d, d);
             Props<double, CASE_LOGN, CASE_R> pr;
             pr.init(a, 0, grp.t);
-            if (rhs) {
+            if (idft) {
+                grp.inverse(fs.Dh, 0);
+            } else if (rhs) {
                 grp.rhs(fs.Dh, c.gN, c.pump);
             } else if (strang) {
                 strang_steps(grp, fs, pr, c, steps);

@@ -226,3 +226,18 @@ def test_increment_unit(builds, tmp_path, logN, R):
     D[:, 0] += 1.2 + 0.4j
     got = run(builds[logN, R], "rk4ip", D, tmp_path, pump=0.5, h=2e-4)
     assert small_mode_errors(D, got, 2e-4, 0.5)[0] <= 2e-21
+
+
+@pytest.mark.parametrize("logN,R", [s for s in shapes() if s[0] >= 4 and s[1] > 2])
+def test_output_0_has_no_bias(builds, tmp_path, logN, R):
+    """Output 0 sums the products with twiddle 1, whose floors are corrected by their mean.  Two strong
+    modes on noise, all modes with sum 0: what a transform returns there is its error, and its mean
+    over the fields has to stay below one field's rounding noise."""
+    N, n = 1 << logN, 256
+    x = np.random.default_rng(N).standard_normal((n, N, 2)).view(complex)[..., 0]
+    x[:, 0] *= 1e6
+    x[:, 3] = 0
+    x[:, 3] = -x.astype(L).sum(axis=1)
+    err = (run(builds[logN, R], "idft", x, tmp_path)[:, 0] - x.astype(L).sum(axis=1)).astype(complex)
+    for e in (err.real, err.imag):
+        assert abs(e.mean()) <= e.std()

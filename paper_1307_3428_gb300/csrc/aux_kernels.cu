@@ -9,10 +9,11 @@ namespace cme {
 
 namespace {
 
-// A complex factor of modulus <= 1 times 2^62 as balanced limbs (cme_fixed.cuh).
-__device__ int4 factor_limbs(double re, double im)
+// A complex factor of modulus <= 1, one + re + i im, times 2^62 as balanced limbs (cme_fixed.cuh).
+// one = 1: re as expm1 gives it, without the rounding of 1 + re to FP64.
+__device__ int4 factor_limbs(double re, double im, int one = 0)
 {
-    const long long C = __double2ll_rn(re * 4611686018427387904.0);
+    const long long C = __double2ll_rn(re * 4611686018427387904.0) + ((long long)one << 62);
     const long long S = __double2ll_rn(im * 4611686018427387904.0);
     return make_int4((int)((unsigned)(C >> 32) + ((unsigned)C >> 31)), (int)C,
                      (int)((unsigned)(S >> 32) + ((unsigned)S >> 31)), (int)S);
@@ -73,8 +74,10 @@ __global__ void prop_kernel(PropArgs a)
     put<V>(a.E, m, make_double2(e1.x + 1.0, e1.y));
     if (a.e1)
         put<V>(a.e1, m, e1);
+    // The fixed-point stages apply E to the state itself, the same E in every step: it keeps the bits
+    // that expm1 gives it, where 1 + expm1 rounded to FP64 is off by up to 2^-54.
     if (a.Ef)
-        reinterpret_cast<int4*>(a.Ef)[m] = factor_limbs(e1.x + 1.0, e1.y);
+        reinterpret_cast<int4*>(a.Ef)[m] = factor_limbs(e1.x, e1.y, 1);
     put<V>(a.e2, m, e2);
     // Strang pump increment over h/2 on the pumped mode (transform position 0):
     //   c = (exp(L_0 h/2) - 1) / L_0 * pump   (h/2 * pump when L_0 = 0)

@@ -1,8 +1,8 @@
 // FP64 transforms in 64-bit fixed point.
 //
 // FP64 instructions run at 1/64 of the FP32 rate on this GPU: a DADD or DFMA holds its scheduler
-// for 64 to 76 cycles, where a 64-bit integer add takes 3 and a 32 x 32 -> 64 multiply 2 (one
-// warp per scheduler).  A transform only adds, subtracts and rotates, and every
+// for 64 to 76 cycles, where a 64-bit integer add takes 3 and a 32 x 32 -> 64 multiply about 4
+// (one warp per scheduler).  A transform only adds, subtracts and rotates, and every
 // intermediate value is a partial sum of unit-modulus multiples of its inputs, so its modulus is
 // at most L1 = sum |x_k|.  The FP64 kernels therefore scale a group's values by one power of two
 // such that this bound fits 61 bits, run the passes on integers, and convert back.  The rounding
@@ -372,11 +372,12 @@ struct FixTransform {
     // the passes from s - 1 on leave free (`up`; lift returns their sum).  Error of the modes below
     // 1e-4 after an RK4IP step of a comb (tests/test_fixed_bounds.py), relative to that of FP64
     // instructions, without and with it: N = 128 at 2 values per thread 1.4 and 0.4, N = 1024 1.7 and
-    // 0.9, N = 2048 1.3 and 1.0, N = 4096 2.2 and 1.55, clusters of 2 ... 8 blocks 1.0 to 2.6 and 0.8 to
+    // 0.9, N = 2048 1.3 and 1.0, N = 4096 2.2 and 1.55, clusters of 2 ... 8 blocks 1.0 to 2.7 and 0.85 to
     // 1.0 at N = 2048, 2.0 to 3.7 and 1.35 to 1.45 at N = 4096; all modes together 1.00.  What is left
     // at N = 4096 is the unit of the Kerr term, set by the envelope's peak, on the samples beside it.
-    // us per RK4IP step without and with: N = 128 x 300 8.6 / 8.7, N = 1024 x 300 36.2 / 36.9,
-    // N = 2048 x 150 45.9 / 46.2, N = 4096 x 150 107.6 / 104.1, x 64 (clusters) 72.6 / 73.1.
+    // us per RK4IP step without and with: N = 128 x 300 8.5 / 8.7, N = 1024 x 300 36.2 / 36.9,
+    // N = 2048 x 150 45.9 / 46.2, N = 4096 x 150 107.7 / 105.0, x 64 (clusters) 72.5 / 72.8; split step
+    // N = 1024 x 76 10.05 / 9.6, N = 2048 x 150 16.7 / 17.1, N = 4096 x 150 35.4 / 36.1.
     CME_HD static constexpr bool lifts(int s)
     {
         return R == 2 ? LOGN == 7 && (s == 3 || s == 5) : (LOGN >= 10 || CLUSTER) && s >= 2;

@@ -27,9 +27,9 @@ using GR = Group<double, CASE_LOGN, CASE_R>;
 constexpr int N = GR::N, P = GR::P, T = P < 32 ? 32 : P, G = T / P;
 inline int host_threads() { return T; }
 
-static int4 limbs(double re, double im)
+static int4 limbs(double re, double im, long long one = 0)
 {
-    const fl r = fsplit(llrint(re * 0x1p62)), i = fsplit(llrint(im * 0x1p62));
+    const fl r = fsplit(llrint(re * 0x1p62) + (one << 62)), i = fsplit(llrint(im * 0x1p62));
     return {r.h, r.l, i.h, i.l};
 }
 
@@ -50,7 +50,7 @@ int main(int argc, char** argv)
     const cx<double> p1 = expm1c(lr * h / 2, li * h / 2), p2 = expm1c(lr * h, li * h);
     for (int k = 0; k < N; ++k) {
         tw[k] = limbs((double)cosl(2 * pi * k / N), (double)sinl(2 * pi * k / N));
-        Ef[k] = limbs(p1.re + 1.0, p1.im);
+        Ef[k] = limbs(p1.re, p1.im, 1);
         E[k] = {p1.re + 1.0, p1.im};
         e1[k] = p1;
         e2[k] = p2;

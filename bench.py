@@ -446,8 +446,8 @@ def large_n_roofline(args, sizes, nsteps, kern_ms, cme, alu):
             "kernel": "large_row_kernel + large_col_kernel (8 per RK4IP step)"}
 
 
-LARGE_SOURCES = ["cme_core.cuh", "cme_step.cuh", "cme_large.cuh", "cme_large_launch.cuh",
-                 "kern_large_fp32.cu"]
+LARGE_SOURCES = ["cme_core.cuh", "cme_fixed.cuh", "cme_step.cuh", "cme_launch.cuh", "cme_large.cuh",
+                 "cme_large_launch.cuh", "kern_large_fp32.cu", "kern_large_fp32_scalar.cu"]
 
 
 def large_source_hash() -> str:

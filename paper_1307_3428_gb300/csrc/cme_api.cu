@@ -135,10 +135,10 @@ bool radix_on_request(int logN, int R, int prec, int inst_per_cta)
 // pay as long as the SMs hold the extra warps side by side: 2 (N <= 128) or 4 (N <= 512, Strang
 // 1024; above, the additional passes cost more) while the group's warps are at most two per
 // scheduler (four schedulers an SM).  RK4IP us per step at 2 / 4 / 8 values, 152 SMs: N = 64 x 1
-// 7.5 / 12.0 / 16.1, x 1216 9.8 / 12.8 / 17.0; N = 128 x 608 11.6 / 12.9 / 19.8, x 1216 (four
-// warps per scheduler at 2, two at 4) 18.6 / 16.2 / 20.0; N = 256 x 608 - / 16.5 / 20.6, x 1216
-// - / 33.1 / 28.1; N = 512 x 256 - / 19.3 / 22.3, x 608 - / 38.6 / 30.0; N = 1024 x 76
-// - / 29.2 / 27.5.  sms = 0: no such information.
+// 7.3 / 10.3 / 16.8, x 1216 9.7 / 10.6 / 16.8; N = 128 x 608 11.6 / 11.5 / 19.5, x 1216 (four
+// warps per scheduler at 2, two at 4) 22.1 / 15.0 / 19.9; N = 256 x 608 - / 16.1 / 20.3, x 1216
+// - / 31.9 / 26.4; N = 512 x 256 - / 18.3 / 22.4, x 608 - / 36.4 / 28.5; N = 1024 x 76
+// - / 28.0 / 28.8.  sms = 0: no such information.
 int default_radix(int logN, int prec, int count = 0, int sms = 0, int method = METHOD_RK4IP)
 {
     if (logN <= 2)
@@ -377,9 +377,9 @@ int plan_batch(cme_batch b, const cme_options& o)
     // stay within ~3.4 per SM (all resident at once), at 8 values per thread; smaller clusters
     // lose to one block.  Measured per RK4IP step,
     // FP32 N = 4096: 16 instances 11.5 -> 5.9 us, 64 instances 11.7 -> 8.2 us, 96 instances
-    // 11.7 -> 15.5 us (not all blocks resident); FP64 N = 4096: 16 instances 108 -> 65 us, 64
-    // instances 108 -> 74 us, 100 instances 109 -> 146 us (C = 4: 166); FP64 N = 2048: 16
-    // instances 52 -> 59 us.  Mixed batches whose one-block plan fills the GPU
+    // 11.7 -> 15.5 us (not all blocks resident); FP64 N = 4096: 16 instances 105 -> 64 us, 64
+    // instances 105 -> 74 us, 100 instances 105 -> 146 us (C = 4: 163); FP64 N = 2048: 16
+    // instances 46 -> 58 us.  Mixed batches whose one-block plan fills the GPU
     // (N = 256 ... 4096 x 64) keep one block per instance: 584 ms per run, against 776 ms with
     // 8-block clusters.
     if (o.cluster == 0 && !any_large && o.persistent != 2 &&   // the work-list kernel has no clusters

@@ -842,7 +842,7 @@ CME_DEV void rk4ip_step_impl(Group<T, LOGN, R, C>& grp, FieldState<T, LOGN, R, C
 // instance: 19.5, 11.7 and 7.2 us.  What bounds it now is one warp per scheduler issuing dependent
 // integer instructions (fixed-latency waits, 1.4 per issue).
 // The error of a step against extended precision on the small modes of a comb (1e-6 beside a
-// pumped mode of 1.3, h = 2e-4): 1.2e-21 at N = 512 and 1.1e-21 at 4096, from 4.9e-21 and 1.6e-21
+// pumped mode of 1.3, h = 2e-4): 1.1e-21 at N = 512 and 1.2e-21 at 4096, from 4.9e-21 and 1.6e-21
 // in FP64 instructions.  It is set by the units of the stage inputs and of the increment, so both
 // keep every bit the bounds leave (fcmul1, not fcmul4, there).
 // park: where the state waits in global memory during the step (groups whose registers and shared
